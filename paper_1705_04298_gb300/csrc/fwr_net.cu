@@ -32,6 +32,7 @@
 
 #include "../../include/fwr.h"
 #include "fwr_internal.h"
+#include "fwr_netgrad.h"
 #include "fwr_plan.h"
 
 namespace fwr {
@@ -39,8 +40,6 @@ namespace net {
 
 constexpr float IN_SCALE = 0.5f;
 constexpr int GRID = 128, LOW = 32, POOL = 4;
-
-typedef __nv_bfloat16 bf16;
 
 // ----------------------------------------------------------------- kernels --
 
@@ -67,10 +66,10 @@ __global__ void k_input(const float* sl, const uint8_t* mask, int n, int off, in
     o[2] = __float2bfloat16(a2 * k);
 }
 
-// extended slopes [F][2][128][128] -> target [F][32][32][2], loss mask [F][32][32]
-__global__ void k_target(const float* ext, const uint8_t* mask, int n, int off, int F, float* T, float* LM) {
+// extended slopes [F][2][128][128] -> target [F][32][32][2], loss mask
+// [F][32][32]; *cnt += the mask's ones (F * 32 * 32 is a multiple of the block)
+__global__ void k_target(const float* ext, const uint8_t* mask, int n, int off, int F, float* T, float* LM, unsigned* cnt) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= F * LOW * LOW) return;
     const int f = idx / (LOW * LOW), Y = (idx / LOW) % LOW, Xc = idx % LOW;
     const float* e = ext + size_t(f) * 2 * GRID * GRID;
     float a0 = 0.f, a1 = 0.f;
@@ -86,7 +85,10 @@ __global__ void k_target(const float* ext, const uint8_t* mask, int n, int off, 
     const float k = IN_SCALE / (POOL * POOL);
     T[2 * idx] = a0 * k;
     T[2 * idx + 1] = a1 * k;
-    LM[idx] = (!pupil && Y != LOW - 1 && Xc != LOW - 1) ? 1.f : 0.f;
+    const bool in = !pupil && Y != LOW - 1 && Xc != LOW - 1;
+    LM[idx] = in ? 1.f : 0.f;
+    const int ones = __syncthreads_count(in);
+    if (threadIdx.x == 0 && ones) atomicAdd(cnt, unsigned(ones));
 }
 
 // 3 x 3 (K = 3) or 1 x 1 (K = 1) convolution. The input is the channel
@@ -293,93 +295,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const bf16* __restrict__
     }
 }
 
-// g <- g * (a > 0)
-__global__ void k_relu_mask(float* g, const bf16* a, size_t n) {
-    const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < n && !(__bfloat162float(a[i]) > 0.f)) g[i] = 0.f;
-}
-
-// dIn[b,y,x,ci] = sum_{co,dy,dx} dZ[b, y-dy+p, x-dx+p, co] W[co][dy][dx][ci]
-template <int K>
-__global__ void k_conv_dgrad(const float* dZ, int cout, int H, int W, const bf16* Wt, int cin, float* dIn) {
-    extern __shared__ float rows[];  // [K][W + 2][cout]
-    const int b = blockIdx.x / H, y = blockIdx.x % H;
-    const int pad = K / 2, RW = W + 2 * pad;
-    for (int i = threadIdx.x; i < K * RW * cout; i += blockDim.x) {
-        const int r = i / (RW * cout), xx = (i / cout) % RW, c = i % cout;
-        const int yy = y - r + pad, xc = xx - pad;  // row r holds dZ at y - r + pad
-        rows[i] = (yy >= 0 && yy < H && xc >= 0 && xc < W) ? dZ[((size_t(b) * H + yy) * W + xc) * cout + c] : 0.f;
-    }
-    __syncthreads();
-    constexpr int XG = 4;
-    const int groups = (W + XG - 1) / XG;
-    for (int t = threadIdx.x; t < cin * groups; t += blockDim.x) {
-        const int ci = t / groups, x0 = (t % groups) * XG;
-        float acc[XG] = {0.f, 0.f, 0.f, 0.f};
-        for (int dy = 0; dy < K; ++dy)
-            for (int dx = 0; dx < K; ++dx)
-                for (int co = 0; co < cout; ++co) {
-                    const float wv = __bfloat162float(Wt[((size_t(co) * K + dy) * K + dx) * cin + ci]);
-#pragma unroll
-                    for (int g = 0; g < XG; ++g) {
-                        const int xc = x0 + g - dx + pad;  // dZ column, shifted by RW offset pad
-                        if (x0 + g < W) acc[g] += wv * rows[(dy * RW + xc + pad) * cout + co];
-                    }
-                }
-        for (int g = 0; g < XG; ++g)
-            if (x0 + g < W) dIn[((size_t(b) * H + y) * W + x0 + g) * cin + ci] = acc[g];
-    }
-}
-
-// dW[co][dy][dx][ci] = sum_{b,y,x} dZ[b,y,x,co] in[b, y+dy-p, x+dx-p, ci];
-// db[co] = sum dZ. One block per (co, dy, dx); threads over (ci, pixel
-// subsets), reduced in shared memory (fixed order).
-template <int K>
-__global__ void k_conv_wgrad(const float* dZ, int cout, const bf16* A, int ca, bool upA, const bf16* Bt, int cb,
-                             int Bn, int H, int W, float* dW, float* db) {
-    const int cin = ca + cb;
-    const int co = blockIdx.x / (K * K), tap = blockIdx.x % (K * K), dy = tap / K, dx = tap % K;
-    const int pad = K / 2;
-    const int nthr = blockDim.x, lanes_c = cin < nthr ? cin : nthr, parts = nthr / lanes_c;
-    const int ci = threadIdx.x % lanes_c, part = threadIdx.x / lanes_c;
-    extern __shared__ float red[];
-    const int P = Bn * H * W;
-    for (int c0 = 0; c0 < cin; c0 += lanes_c) {
-        const int c = c0 + ci;
-        float acc = 0.f, accb = 0.f;
-        if (part < parts && c < cin) {
-            for (int p = part; p < P; p += parts) {
-                const int b = p / (H * W), y = (p / W) % H, x = p % W;
-                const float g = dZ[size_t(p) * cout + co];
-                if (c0 == 0 && ci == 0 && tap == 0) accb += g;
-                const int yy = y + dy - pad, xc = x + dx - pad;
-                if (yy < 0 || yy >= H || xc < 0 || xc >= W) continue;
-                float v;
-                if (c < ca) {
-                    v = upA ? __bfloat162float(A[((size_t(b) * (H / 2) + yy / 2) * (W / 2) + xc / 2) * ca + c])
-                            : __bfloat162float(A[((size_t(b) * H + yy) * W + xc) * ca + c]);
-                } else {
-                    v = __bfloat162float(Bt[((size_t(b) * H + yy) * W + xc) * cb + (c - ca)]);
-                }
-                acc += g * v;
-            }
-        }
-        red[threadIdx.x] = acc;
-        red[nthr + threadIdx.x] = accb;
-        __syncthreads();
-        if (part == 0 && c < cin) {
-            float s = 0.f, sb = 0.f;
-            for (int q = 0; q < parts; ++q) {
-                s += red[q * lanes_c + ci];
-                sb += red[nthr + q * lanes_c + ci];
-            }
-            dW[((size_t(co) * K + dy) * K + dx) * cin + c] = s;
-            if (c0 == 0 && ci == 0 && tap == 0) db[co] = sb;
-        }
-        __syncthreads();
-    }
-}
-
 __global__ void k_avgpool(const bf16* in, int Bn, int H, int W, int C, bf16* out) {
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int Ho = H / 2, Wo = W / 2;
@@ -391,61 +306,13 @@ __global__ void k_avgpool(const bf16* in, int Bn, int H, int W, int C, bf16* out
     out[i] = __float2bfloat16(0.25f * s);
 }
 
-// dIn (H x W) += pool^T(dOut)
-__global__ void k_avgpool_bwd_add(const float* dOut, int Bn, int H, int W, int C, float* dIn) {
+// dIn (H x W) <- (dIn + pool^T(dOut)), zeroed where the pooled activation act is not positive
+__global__ void k_avgpool_bwd_add(const float* dOut, const bf16* act, int Bn, int H, int W, int C, float* dIn) {
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= size_t(Bn) * H * W * C) return;
     const int c = i % C, x = (i / C) % W, y = (i / (size_t(C) * W)) % H, b = i / (size_t(C) * W * H);
-    dIn[i] += 0.25f * dOut[((size_t(b) * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c];
-}
-
-// dCat [B,H,W,ca+cb] -> dLow [B,H/2,W/2,ca] = up^T(dCat[..., :ca]); dSkip (+)= dCat[..., ca:]
-__global__ void k_split_concat(const float* dCat, int Bn, int H, int W, int ca, int cb, float* dLow, float* dSkip) {
-    const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int C = ca + cb;
-    const int Hl = H / 2, Wl = W / 2;
-    if (i < size_t(Bn) * Hl * Wl * ca) {
-        const int c = i % ca, x = (i / ca) % Wl, y = (i / (size_t(ca) * Wl)) % Hl, b = i / (size_t(ca) * Wl * Hl);
-        float s = 0.f;
-        for (int a = 0; a < 2; ++a)
-            for (int d = 0; d < 2; ++d) s += dCat[((size_t(b) * H + 2 * y + a) * W + 2 * x + d) * C + c];
-        dLow[i] = s;
-    }
-    if (i < size_t(Bn) * H * W * cb) {
-        const int c = i % cb;
-        const size_t p = i / cb;
-        dSkip[i] = dCat[p * C + ca + c];
-    }
-}
-
-// masked MSE: loss += sum m (p - t)^2 / cnt ; dP = 2 m (p - t) / cnt
-__global__ void k_loss(const float* pred, const float* T, const float* LM, int npix, float inv_cnt, float* dP,
-                       float* loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (i < npix) {
-        const float m = LM[i];
-        const float d0 = (pred[2 * i] - T[2 * i]) * m, d1 = (pred[2 * i + 1] - T[2 * i + 1]) * m;
-        dP[2 * i] = 2.f * d0 * inv_cnt;
-        dP[2 * i + 1] = 2.f * d1 * inv_cnt;
-        l = (d0 * d0 + d1 * d1) * inv_cnt;
-    }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
-}
-
-__global__ void k_sum(const float* v, int n, float* out) {
-    float s = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ float part[32];
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int(blockDim.x) + 31) / 32; ++w) t += part[w];
-        *out = t;
-    }
+    const float g = dIn[i] + 0.25f * dOut[((size_t(b) * (H / 2) + y / 2) * (W / 2) + x / 2) * C + c];
+    dIn[i] = __bfloat162float(act[i]) > 0.f ? g : 0.f;
 }
 
 __global__ void k_adam(float* w, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float eps,
@@ -507,8 +374,11 @@ struct fwr_net {
     std::vector<bf16*> act;
     std::vector<float*> grad;
     bf16 *X = nullptr, *pool1 = nullptr, *pool2 = nullptr, *pool3 = nullptr;
-    float *pred = nullptr, *dpred = nullptr, *T = nullptr, *LM = nullptr, *loss = nullptr, *cnt = nullptr;
-    float *dcat = nullptr, *dtmp = nullptr, *dpool = nullptr;
+    float *pred = nullptr, *T = nullptr, *LM = nullptr, *loss = nullptr;
+    unsigned* cnt = nullptr;    // ones of the loss mask
+    float *dpool = nullptr;
+    float* gws = nullptr;       // per-CTA weight-gradient sums
+    int sms = 0;
 };
 
 namespace {
@@ -620,83 +490,58 @@ cudaError_t forward(fwr_net* n, int Bn, cudaStream_t s) {
     return conv_fwd(n, 14, a[13], nullptr, Bn, nullptr, n->pred, s);
 }
 
-// backward of one conv layer: dZ = g (relu-masked by the caller); writes dW,
-// db into G and dIn (concatenated input gradient) into din
-cudaError_t conv_bwd(fwr_net* n, int li, const float* dZ, const bf16* A, const bf16* B, int Bn, float* din,
-                     cudaStream_t s) {
+// backward of one 3 x 3 layer: dZ = the gradient of its output before the
+// ReLU; writes dW, db into G and the input gradient (conv_dgrad) into din and lo
+cudaError_t conv_bwd(fwr_net* n, int li, const float* dZ, const bf16* A, const bf16* B, int Bn, const bf16* act,
+                     float* din, float* lo, const bf16* lo_act, cudaStream_t s) {
     const Layer& L = n->layers[li];
-    const int cin = L.ca + L.cb, RW = L.H + 2 * (L.k / 2);
-    const int thr = 256;
-    if (L.k == 3) {
-        k_conv_wgrad<3><<<L.cout * 9, thr, 2 * thr * sizeof(float), s>>>(dZ, L.cout, A, L.ca, L.upA, B, L.cb, Bn, L.H,
-                                                                          L.H, n->G + L.woff, n->G + L.boff);
-        if (din)
-            k_conv_dgrad<3><<<Bn * L.H, 256, size_t(3) * RW * L.cout * sizeof(float), s>>>(
-                dZ, L.cout, L.H, L.H, n->Wb + L.woff, cin, din);
-    } else {
-        k_conv_wgrad<1><<<L.cout, thr, 2 * thr * sizeof(float), s>>>(dZ, L.cout, A, L.ca, L.upA, B, L.cb, Bn, L.H,
-                                                                      L.H, n->G + L.woff, n->G + L.boff);
-        if (din)
-            k_conv_dgrad<1><<<Bn * L.H, 256, size_t(1) * RW * L.cout * sizeof(float), s>>>(
-                dZ, L.cout, L.H, L.H, n->Wb + L.woff, cin, din);
-    }
-    return cudaGetLastError();
+    const ConvBwd c{L.ca, L.cb, L.cout, L.H, L.upA, A, B};
+    cudaError_t e = conv_wgrad(c, dZ, Bn, n->gws, n->G + L.woff, n->sms, s);
+    if (e == cudaSuccess && din) e = conv_dgrad(c, dZ, n->Wb + L.woff, Bn, act, din, lo, lo_act, s);
+    return e;
 }
 
-void relu_mask(float* g, const bf16* a, size_t cnt, cudaStream_t s) {
-    k_relu_mask<<<blocks(cnt, 256), 256, 0, s>>>(g, a, cnt);
-}
-
-// backward of the whole network from n->dpred; gradients into n->G
+// loss and backward of the whole network from n->pred; gradients into n->G.
+// Every gradient of an activation is stored with the ReLU's mask applied by
+// the kernel that completes it.
 cudaError_t backward(fwr_net* n, int Bn, cudaStream_t s) {
     bf16** a = n->act.data();
     float** g = n->grad.data();
-    const int w1 = n->w, w2 = 2 * n->w, w3 = 4 * n->w, w4 = 4 * n->w;
+    const int w1 = n->w, w2 = 2 * n->w, w3 = 4 * n->w;
     auto px = [&](int H, int C) { return size_t(Bn) * H * H * C; };
     cudaError_t e;
-    // out: 1x1, no ReLU
-    if ((e = conv_bwd(n, 14, n->dpred, a[13], nullptr, Bn, g[13], s)) != cudaSuccess) return e;
+    // loss and out: 1x1, no ReLU
+    const Layer& lo = n->layers[14];
+    if ((e = out_backward(n->pred, n->T, n->LM, n->cnt, Bn * LOW * LOW, w1, a[13], n->Wb + lo.woff, g[13], n->gws,
+                          n->G + lo.woff, n->loss, n->sms, s)) != cudaSuccess)
+        return e;
     // d1b, d1a (input concat [up(d2b) w2 | s1 w1] at 32)
-    relu_mask(g[13], a[13], px(32, w1), s);
-    if ((e = conv_bwd(n, 13, g[13], a[12], nullptr, Bn, g[12], s)) != cudaSuccess) return e;
-    relu_mask(g[12], a[12], px(32, w1), s);
-    if ((e = conv_bwd(n, 12, g[12], a[11], a[1], Bn, n->dcat, s)) != cudaSuccess) return e;
-    k_split_concat<<<blocks(px(32, w1 + w2), 256), 256, 0, s>>>(n->dcat, Bn, 32, 32, w2, w1, g[11], g[1]);
+    if ((e = conv_bwd(n, 13, g[13], a[12], nullptr, Bn, a[12], g[12], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 12, g[12], a[11], a[1], Bn, nullptr, g[1], g[11], a[11], s)) != cudaSuccess) return e;
     // d2b, d2a (concat [up(d3b) w3 | s2 w2] at 16)
-    relu_mask(g[11], a[11], px(16, w2), s);
-    if ((e = conv_bwd(n, 11, g[11], a[10], nullptr, Bn, g[10], s)) != cudaSuccess) return e;
-    relu_mask(g[10], a[10], px(16, w2), s);
-    if ((e = conv_bwd(n, 10, g[10], a[9], a[3], Bn, n->dcat, s)) != cudaSuccess) return e;
-    k_split_concat<<<blocks(px(16, w2 + w3), 256), 256, 0, s>>>(n->dcat, Bn, 16, 16, w3, w2, g[9], g[3]);
+    if ((e = conv_bwd(n, 11, g[11], a[10], nullptr, Bn, a[10], g[10], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 10, g[10], a[9], a[3], Bn, nullptr, g[3], g[9], a[9], s)) != cudaSuccess) return e;
     // d3b, d3a (concat [up(bb) w4 | s3 w3] at 8)
-    relu_mask(g[9], a[9], px(8, w3), s);
-    if ((e = conv_bwd(n, 9, g[9], a[8], nullptr, Bn, g[8], s)) != cudaSuccess) return e;
-    relu_mask(g[8], a[8], px(8, w3), s);
-    if ((e = conv_bwd(n, 8, g[8], a[7], a[5], Bn, n->dcat, s)) != cudaSuccess) return e;
-    k_split_concat<<<blocks(px(8, w3 + w4), 256), 256, 0, s>>>(n->dcat, Bn, 8, 8, w4, w3, g[7], g[5]);
+    if ((e = conv_bwd(n, 9, g[9], a[8], nullptr, Bn, a[8], g[8], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 8, g[8], a[7], a[5], Bn, nullptr, g[5], g[7], a[7], s)) != cudaSuccess) return e;
     // bottleneck at 4
-    relu_mask(g[7], a[7], px(4, w4), s);
-    if ((e = conv_bwd(n, 7, g[7], a[6], nullptr, Bn, g[6], s)) != cudaSuccess) return e;
-    relu_mask(g[6], a[6], px(4, w4), s);
-    if ((e = conv_bwd(n, 6, g[6], n->pool3, nullptr, Bn, n->dpool, s)) != cudaSuccess) return e;
-    k_avgpool_bwd_add<<<blocks(px(8, w3), 256), 256, 0, s>>>(n->dpool, Bn, 8, 8, w3, g[5]);
+    if ((e = conv_bwd(n, 7, g[7], a[6], nullptr, Bn, a[6], g[6], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 6, g[6], n->pool3, nullptr, Bn, nullptr, n->dpool, nullptr, nullptr, s)) != cudaSuccess)
+        return e;
+    k_avgpool_bwd_add<<<blocks(px(8, w3), 256), 256, 0, s>>>(n->dpool, a[5], Bn, 8, 8, w3, g[5]);
     // encoder level 3 (8)
-    relu_mask(g[5], a[5], px(8, w3), s);
-    if ((e = conv_bwd(n, 5, g[5], a[4], nullptr, Bn, g[4], s)) != cudaSuccess) return e;
-    relu_mask(g[4], a[4], px(8, w3), s);
-    if ((e = conv_bwd(n, 4, g[4], n->pool2, nullptr, Bn, n->dpool, s)) != cudaSuccess) return e;
-    k_avgpool_bwd_add<<<blocks(px(16, w2), 256), 256, 0, s>>>(n->dpool, Bn, 16, 16, w2, g[3]);
+    if ((e = conv_bwd(n, 5, g[5], a[4], nullptr, Bn, a[4], g[4], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 4, g[4], n->pool2, nullptr, Bn, nullptr, n->dpool, nullptr, nullptr, s)) != cudaSuccess)
+        return e;
+    k_avgpool_bwd_add<<<blocks(px(16, w2), 256), 256, 0, s>>>(n->dpool, a[3], Bn, 16, 16, w2, g[3]);
     // level 2 (16)
-    relu_mask(g[3], a[3], px(16, w2), s);
-    if ((e = conv_bwd(n, 3, g[3], a[2], nullptr, Bn, g[2], s)) != cudaSuccess) return e;
-    relu_mask(g[2], a[2], px(16, w2), s);
-    if ((e = conv_bwd(n, 2, g[2], n->pool1, nullptr, Bn, n->dpool, s)) != cudaSuccess) return e;
-    k_avgpool_bwd_add<<<blocks(px(32, w1), 256), 256, 0, s>>>(n->dpool, Bn, 32, 32, w1, g[1]);
+    if ((e = conv_bwd(n, 3, g[3], a[2], nullptr, Bn, a[2], g[2], nullptr, nullptr, s)) != cudaSuccess) return e;
+    if ((e = conv_bwd(n, 2, g[2], n->pool1, nullptr, Bn, nullptr, n->dpool, nullptr, nullptr, s)) != cudaSuccess)
+        return e;
+    k_avgpool_bwd_add<<<blocks(px(32, w1), 256), 256, 0, s>>>(n->dpool, a[1], Bn, 32, 32, w1, g[1]);
     // level 1 (32)
-    relu_mask(g[1], a[1], px(32, w1), s);
-    if ((e = conv_bwd(n, 1, g[1], a[0], nullptr, Bn, g[0], s)) != cudaSuccess) return e;
-    relu_mask(g[0], a[0], px(32, w1), s);
-    return conv_bwd(n, 0, g[0], n->X, nullptr, Bn, nullptr, s);
+    if ((e = conv_bwd(n, 1, g[1], a[0], nullptr, Bn, a[0], g[0], nullptr, nullptr, s)) != cudaSuccess) return e;
+    return conv_bwd(n, 0, g[0], n->X, nullptr, Bn, nullptr, nullptr, nullptr, nullptr, s);
 }
 
 void free_net(fwr_net* n) {
@@ -713,14 +558,12 @@ void free_net(fwr_net* n) {
     cudaFree(n->pool2);
     cudaFree(n->pool3);
     cudaFree(n->pred);
-    cudaFree(n->dpred);
     cudaFree(n->T);
     cudaFree(n->LM);
     cudaFree(n->loss);
     cudaFree(n->cnt);
-    cudaFree(n->dcat);
-    cudaFree(n->dtmp);
     cudaFree(n->dpool);
+    cudaFree(n->gws);
     delete n;
 }
 
@@ -773,18 +616,24 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
         n->act.push_back(a);
         n->grad.push_back(g);
     }
-    const int w1 = width, w2 = 2 * width, w3 = 4 * width, w4 = 4 * width;
+    const int w1 = width, w2 = 2 * width, w3 = 4 * width;
     balloc(&n->X, B * 32 * 32 * 3);
     balloc(&n->pool1, B * 16 * 16 * w1);
     balloc(&n->pool2, B * 8 * 8 * w2);
     balloc(&n->pool3, B * 4 * 4 * w3);
     falloc(&n->pred, B * 32 * 32 * 2);
-    falloc(&n->dpred, B * 32 * 32 * 2);
     falloc(&n->T, B * 32 * 32 * 2);
     falloc(&n->LM, B * 32 * 32);
     falloc(&n->loss, 1);
-    falloc(&n->cnt, 1);
-    falloc(&n->dcat, B * 32 * 32 * size_t(w1 + w2 + w3 + w4));
+    if (e == cudaSuccess) e = cudaMalloc(&n->cnt, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, n->device);
+    size_t gws = out_ws_floats(width, n->sms);
+    for (const Layer& L : n->layers) {
+        if (L.k != 3) continue;
+        gws = std::max(gws, wgrad_ws_floats(L.ca + L.cb, L.cout, L.H, n->sms));
+        if (e == cudaSuccess && !netgrad_prepare(L.ca + L.cb, L.cout, L.H)) e = cudaErrorInvalidValue;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&n->gws, gws * sizeof(float));
     falloc(&n->dpool, B * 16 * 16 * w1 + B * 8 * 8 * w2 + B * 4 * 4 * w3);
     if (e == cudaSuccess) {
         std::vector<float> h(n->nparam, 0.f);
@@ -796,16 +645,13 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }
     // the convolution kernels stage K rows of (H + 2) pixels x channels as floats
-    size_t fwd_smem = 0, dgrad_smem = 0;
-    for (const Layer& L : n->layers) {
-        const size_t rw = size_t(L.H + 2 * (L.k / 2)) * L.k * sizeof(float);
-        fwd_smem = std::max(fwd_smem, rw * (L.ca + L.cb));
-        dgrad_smem = std::max(dgrad_smem, rw * L.cout);
-    }
+    size_t fwd_smem = 0;
+    for (const Layer& L : n->layers)
+        fwd_smem = std::max(fwd_smem, size_t(L.H + 2 * (L.k / 2)) * L.k * sizeof(float) * (L.ca + L.cb));
     size_t tc_smem = 0;
     for (const Layer& L : n->layers)
         if (L.tc) tc_smem = std::max(tc_smem, tc_smem_bytes(L.H, L.ca + L.cb));
-    if (fwd_smem > 227 * 1024 || dgrad_smem > 227 * 1024) e = cudaErrorInvalidValue;
+    if (fwd_smem > 227 * 1024) e = cudaErrorInvalidValue;
     if (tc_smem > 227 * 1024) {
         for (Layer& L : n->layers) L.tc = false;
         tc_smem = 0;
@@ -819,8 +665,6 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
     }
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_conv_fwd<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fwd_smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_conv_dgrad<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dgrad_smem));
     if (e != cudaSuccess) {
         free_net(n);
         return fwr::cuda_fail(e, "fwr_net_create");
@@ -889,23 +733,13 @@ fwr_status fwr_net_gradients(fwr_net* n, const fwr_plan* p, const float* slopes,
     if (!n || !geometry_ok(p) || F < 1 || F > n->max_batch || !slopes || !target_ext) return FWR_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = prepare(n, p, slopes, F, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(n->cnt, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
         k_target<<<blocks(size_t(F) * LOW * LOW, 256), 256, 0, s>>>(target_ext, p->d_mask, p->n, p->off, F, n->T,
-                                                                     n->LM);
-        k_sum<<<1, 1024, 0, s>>>(n->LM, F * LOW * LOW, n->cnt);
+                                                                     n->LM, n->cnt);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = forward(n, F, s);
-    float cnt = 0.f;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, n->cnt, sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) {
-        cudaMemsetAsync(n->loss, 0, sizeof(float), s);
-        const int npix = F * LOW * LOW;
-        k_loss<<<blocks(npix, 256), 256, 0, s>>>(n->pred, n->T, n->LM, npix, 1.f / fmaxf(1.f, 2.f * cnt), n->dpred,
-                                                  n->loss);
-        e = cudaGetLastError();
-    }
     if (e == cudaSuccess) e = backward(n, F, s);
     if (e == cudaSuccess && loss_host) e = cudaMemcpyAsync(loss_host, n->loss, sizeof(float), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && grad_host)

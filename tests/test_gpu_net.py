@@ -136,3 +136,23 @@ def test_training_lowers_the_loss(fwr):
     for _ in range(60):
         last = net.train_step(plan, s, ext, 1e-3)
     assert np.isfinite(last) and last < 0.8 * first, (first, last)
+
+
+@pytest.mark.parametrize("w,F", [(1, 1), (5, 3), (8, 17), (32, 2)])
+def test_gradients_at_other_widths(fwr, w, F):
+    """Widths whose channel counts leave remainders in the backward kernels'
+    register tiles (8 x 4 and 8 channels) and vector loads, and a width whose
+    output tiles span several CTAs; batches that end inside a CTA's images.
+    The bounds are those of the activations' BF16 storage (2^-9 relative per
+    rounding, 14 layers deep), as above."""
+    plan, sl, mask, off, ext, params = setup_problem(fwr, w, F, 33)
+    net = fwr.Net(w, max(F, 4), params)
+    s = torch.tensor(sl, dtype=torch.float32, device="cuda")
+    e = torch.tensor(ext, dtype=torch.float32, device="cuda")
+    loss, g = net.gradients(plan, s, e)
+    loss2, g2 = net.gradients(plan, s, e)
+    assert loss == loss2 and np.array_equal(g, g2)
+    out_o, loss_o, g_o = oracle_run(params, w, sl, mask, off, ext)
+    assert abs(loss - loss_o) <= 2e-2 * abs(loss_o)
+    rel = np.linalg.norm(g - g_o) / np.linalg.norm(g_o)
+    assert rel <= 5e-2, rel
