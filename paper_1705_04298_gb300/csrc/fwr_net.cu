@@ -497,7 +497,7 @@ cudaError_t conv_bwd(fwr_net* n, int li, const float* dZ, const bf16* A, const b
     const Layer& L = n->layers[li];
     const ConvBwd c{L.ca, L.cb, L.cout, L.H, L.upA, A, B};
     cudaError_t e = conv_wgrad(c, dZ, Bn, n->gws, n->G + L.woff, n->sms, s);
-    if (e == cudaSuccess && din) e = conv_dgrad(c, dZ, n->Wb + L.woff, Bn, act, din, lo, lo_act, s);
+    if (e == cudaSuccess && din) e = conv_dgrad(c, dZ, n->Wb + L.woff, Bn, act, din, lo, lo_act, n->sms, s);
     return e;
 }
 

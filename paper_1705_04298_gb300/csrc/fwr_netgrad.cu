@@ -8,7 +8,7 @@
 // Each thread keeps a register tile whose operands come from shared memory in
 // 16-byte loads, few loads per FMA. Measured on 256 images at width 16, the
 // whole gradient call: 90.6 ms with scalar kernels (one block per output
-// channel and tap, operands from global memory), 3.2 ms with these.
+// channel and tap, operands from global memory), 2.5 ms with these.
 
 #include <stdint.h>
 
@@ -61,7 +61,15 @@ constexpr size_t WGRAD_SMEM = 108 * 1024;
 // memory and every CTA (a chunk of rows) writes its sums to ws; k_reduce adds
 // the chunks in order, so the result does not depend on timing.
 
+// i / d for 0 <= i < 2^16 and 1 <= d < 2^16 as one multiply
+struct FastDiv {
+    unsigned d, m;
+};
+FastDiv fast_div(int d) { return FastDiv{unsigned(d), unsigned(((1ull << 32) + d - 1) / d)}; }
+__device__ __forceinline__ int div_by(int i, FastDiv f) { return f.d == 1u ? i : int(__umulhi(unsigned(i), f.m)); }
+
 struct WgradShape {
+    FastDiv by_ncib, by_q;
     int cin4, cout8, ncib, ncob, T, ny, TG, S, threads, RS, zrow, irow;
     size_t smem;
 };
@@ -72,6 +80,8 @@ WgradShape wgrad_shape(int cin, int cout, int H) {
     w.cout8 = (cout + 7) / 8 * 8;
     w.ncib = w.cin4 / 4;
     w.ncob = w.cout8 / 8;
+    w.by_ncib = fast_div(w.ncib);
+    w.by_q = fast_div(std::max(1, H * cout / 4));
     w.T = w.ncib * w.ncob * 3;
     w.ny = (w.T + THREADS - 1) / THREADS;
     w.TG = (w.T + w.ny - 1) / w.ny;
@@ -99,13 +109,15 @@ int wgrad_rows(const WgradShape& w, long long rows, int sms) {
     return int(r);
 }
 
+template <int H>
 __global__ void __launch_bounds__(THREADS)
 k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int ca, int upA,
-         const bf16* __restrict__ Bt, int cb, int H, int rows, int rows_cta, WgradShape w, float* __restrict__ ws) {
+         const bf16* __restrict__ Bt, int cb, int rows, int rows_cta, WgradShape w, float* __restrict__ ws) {
     extern __shared__ __align__(16) float sm[];
     float* const zs = sm;                      // [RS][H][cout8]
     float* const is = sm + size_t(w.RS) * w.zrow;  // [RS + 2][H + 2][cin4]
-    const int W = H, cin = ca + cb;
+    constexpr int W = H;
+    const int cin = ca + cb;
     const int tid = threadIdx.x;
     const int s = tid / w.TG, t = blockIdx.y * w.TG + tid % w.TG;
     const bool active = s < w.S && t < w.T;
@@ -129,8 +141,9 @@ k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int
         // dZ rows (contiguous in memory)
         if ((cout & 7) == 0) {
             const int q = W * cout / 4;
+#pragma unroll 4
             for (int i = tid; i < nr * q; i += blockDim.x) {
-                const int r = i / q, c = i - r * q;
+                const int r = div_by(i, w.by_q), c = i - r * q;
                 reinterpret_cast<float4*>(zs + r * w.zrow)[c] =
                     __ldg(reinterpret_cast<const float4*>(dZ + size_t(r0 + r) * W * cout) + c);
             }
@@ -142,8 +155,9 @@ k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int
         }
         // input rows r0 - 1 .. r0 + nr, one zero column on each side
         const bool vec = (ca & 3) == 0 && (cb & 3) == 0;
+#pragma unroll 4
         for (int i = tid; i < (nr + 2) * (W + 2) * w.ncib; i += blockDim.x) {
-            const int c = (i % w.ncib) * 4, xx = (i / w.ncib) % (W + 2), r = i / (w.ncib * (W + 2));
+            const int q = div_by(i, w.by_ncib), c = (i - q * w.ncib) * 4, xx = q % (W + 2), r = q / (W + 2);
             const int gr = r0 - 1 + r, x = xx - 1;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (gr >= 0 && gr < rows && x >= 0 && x < W) {
@@ -308,17 +322,16 @@ constexpr int DG_CO = 16;
 constexpr size_t DGRAD_SMEM = 100 * 1024;
 
 struct DgradShape {
-    int cb, ny, pairs, threads, slots, portion;  // portion: row pairs per image part
+    int cb, ny, pairs, S, threads, slots, portion;  // portion: row pairs per image part
     size_t smem;
 };
 
-DgradShape dgrad_shape(int cin, int H) {
+DgradShape dgrad_shape(int cin, int H, long long total_pairs, int sms) {
     DgradShape d;
     const int blk = (cin + 7) / 8;
     d.ny = (blk + 7) / 8;
     d.cb = (blk + d.ny - 1) / d.ny;
     const int per_pair = H / 4;  // tiles of a row pair
-    d.pairs = 1;
     const int img = H / 2;
     auto slots = [&](int pairs) {
         const int portion = pairs < img ? pairs : img;
@@ -329,24 +342,37 @@ DgradShape dgrad_shape(int cin, int H) {
     };
     // 128 to 254 threads (several CTAs fit an SM's registers) unless dZ's rows
     // would leave room for one CTA only (few channels on the smallest images)
+    d.pairs = 1;
     while (d.cb * per_pair * d.pairs < 128 && bytes(2 * d.pairs) <= DGRAD_SMEM) d.pairs *= 2;
+    // the small images' layers have few tiles: fewer per CTA, each shared by S
+    // threads over the output channels, until there are two CTAs per SM (256
+    // images of 8 x 8 and 64 channels: 161 us with S = 1, 64 with 4)
+    d.S = 1;
+    while (d.S < 8 && (total_pairs + d.pairs - 1) / d.pairs * d.ny < 2 * sms) {
+        if (d.pairs > 1) d.pairs /= 2;
+        else if (2 * d.S * d.cb * per_pair > THREADS) break;
+        d.S *= 2;
+    }
     d.portion = d.pairs < img ? d.pairs : img;
     d.slots = slots(d.pairs);
-    d.threads = d.cb * per_pair * d.pairs;
-    d.smem = bytes(d.pairs);
+    d.threads = d.cb * per_pair * d.pairs * d.S;
+    d.smem = std::max(bytes(d.pairs), size_t(d.threads / 2) * 33 * sizeof(u64));
     return d;
 }
 
+template <int H>
 __global__ void __launch_bounds__(THREADS)
-k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, int ca, int cb2, int H, int total_pairs,
+k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, int ca, int cb2, int total_pairs,
          DgradShape d, const bf16* __restrict__ act, float* __restrict__ dIn, float* __restrict__ lo,
          const bf16* __restrict__ lo_act) {
     extern __shared__ __align__(16) float sm[];
-    const int W = H, cin = ca + cb2, ZS = W + 8, n8 = 8 * d.cb;
+    constexpr int W = H, ZS = W + 8;
+    const int cin = ca + cb2, n8 = 8 * d.cb;
     float* const zs = sm;                                     // [slots][DG_CO][ZS], column x at 4 + x
     float* const wsm = sm + size_t(d.slots) * DG_CO * ZS;     // [DG_CO][9][n8]
-    const int tid = threadIdx.x, img = H / 2;
-    const int cib = tid % d.cb, tile = tid / d.cb;
+    constexpr int img = H / 2;
+    const int tid = threadIdx.x, tt = blockDim.x / d.S, sp = tid / tt, tl = tid - sp * tt;
+    const int cib = tl % d.cb, tile = tl / d.cb;
     const int xt = tile % (W / 4), pr = tile / (W / 4);       // tile column, row pair in the CTA
     const int pair0 = blockIdx.x * d.pairs, ci0 = blockIdx.y * n8;
     const int part = pr / d.portion, slot0 = part * (2 * d.portion + 2) + 2 * (pr - part * d.portion);
@@ -361,6 +387,7 @@ k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, in
     for (int c0 = 0; c0 < cout; c0 += DG_CO) {
         const int nc = min(DG_CO, cout - c0);
         __syncthreads();
+#pragma unroll 4
         for (int i = tid; i < d.slots * (DG_CO / 4) * W; i += blockDim.x) {
             const int x = i % W, c4 = (i / W) % (DG_CO / 4), slot = i / (W * (DG_CO / 4));
             const int p = slot / (2 * d.portion + 2), j = slot - p * (2 * d.portion + 2);
@@ -384,15 +411,17 @@ k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, in
             o[2 * ZS] = v.z;
             o[3 * ZS] = v.w;
         }
-        for (int i = tid; i < nc * 9 * n8; i += blockDim.x) {
-            const int c = i % n8, ct = i / n8;
-            wsm[i] = ci0 + c < cin ? __bfloat162float(Wt[(size_t(c0) * 9 + ct) * cin + ci0 + c]) : 0.f;
+        // weight rows (output channel, tap): two rows per warp at a time, 16 lanes each
+        for (int ct = tid >> 4; ct < nc * 9; ct += blockDim.x >> 4) {
+            const bf16* src = Wt + (size_t(c0) * 9 + ct) * cin + ci0;
+#pragma unroll 4
+            for (int c = tid & 15; c < n8; c += 16) wsm[ct * n8 + c] = ci0 + c < cin ? __bfloat162float(src[c]) : 0.f;
         }
         __syncthreads();
-        const float* zp = zs + slot0 * DG_CO * ZS + 4 + 4 * xt;
-        const float* wp = wsm + 4 * cib;
+        const float* zp = zs + (slot0 * DG_CO + sp) * ZS + 4 + 4 * xt;
+        const float* wp = wsm + sp * 9 * n8 + 4 * cib;
 #pragma unroll 1
-        for (int co = 0; co < nc; ++co, zp += ZS, wp += 9 * n8) {
+        for (int co = sp; co < nc; co += d.S, zp += d.S * ZS, wp += d.S * 9 * n8) {
             u64 z[4][6];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -421,8 +450,28 @@ k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, in
             }
         }
     }
+    // sum the S copies, pairwise halves
+    for (int n = d.S; n > 1; n /= 2) {
+        u64* const red = reinterpret_cast<u64*>(sm);  // [copy][tile][33]
+        __syncthreads();
+        if (sp >= n / 2 && sp < n) {
+            u64* o = red + size_t((sp - n / 2) * tt + tl) * 33;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[4 * i + j] = acc[i][j];
+        }
+        __syncthreads();
+        if (sp < n / 2) {
+            const u64* o = red + size_t(sp * tt + tl) * 33;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = add2(acc[i][j], o[4 * i + j]);
+        }
+    }
     const int gp = pair0 + pr;
-    if (gp >= total_pairs) return;
+    if (sp != 0 || gp >= total_pairs) return;
     const int b = gp / img, y0 = 2 * (gp - b * img), x0 = 4 * xt;
     const bool vec = (cin & 3) == 0 && (ca & 3) == 0;
 #pragma unroll
@@ -555,19 +604,21 @@ cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, flo
     const int cin = L.ca + L.cb, rows = Bn * L.H;
     const WgradShape w = wgrad_shape(cin, L.cout, L.H);
     const int rc = wgrad_rows(w, rows, sms), chunks = (rows + rc - 1) / rc;
-    k_wgrad3<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, L.H, rows,
-                                                          rc, w, ws);
+    auto kern = L.H == 32 ? k_wgrad3<32> : L.H == 16 ? k_wgrad3<16> : L.H == 8 ? k_wgrad3<8> : k_wgrad3<4>;
+    kern<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
+                                                       ws);
     const int n = L.cout * 9 * cin + L.cout;
     k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, chunks, n, g, nullptr);
     return cudaGetLastError();
 }
 
 cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
-                       float* lo, const bf16* lo_act, cudaStream_t s) {
-    const DgradShape d = dgrad_shape(L.ca + L.cb, L.H);
+                       float* lo, const bf16* lo_act, int sms, cudaStream_t s) {
     const int pairs = Bn * (L.H / 2);
-    k_dgrad3<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.threads, d.smem, s>>>(
-        dZ, L.cout, Wt, L.ca, L.cb, L.H, pairs, d, act, dIn, lo, lo_act);
+    const DgradShape d = dgrad_shape(L.ca + L.cb, L.H, pairs, sms);
+    auto kern = L.H == 32 ? k_dgrad3<32> : L.H == 16 ? k_dgrad3<16> : L.H == 8 ? k_dgrad3<8> : k_dgrad3<4>;
+    kern<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.threads, d.smem, s>>>(dZ, L.cout, Wt, L.ca, L.cb, pairs, d,
+                                                                               act, dIn, lo, lo_act);
     return cudaGetLastError();
 }
 
@@ -585,11 +636,15 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
 }
 
 bool netgrad_prepare(int cin, int cout, int H) {
-    const size_t most = std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H).smem);
     const int lim = 227 * 1024;
-    if (most > size_t(lim)) return false;
-    return cudaFuncSetAttribute(k_wgrad3, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess &&
-           cudaFuncSetAttribute(k_dgrad3, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
+    if (H != 32 && H != 16 && H != 8 && H != 4) return false;
+    if (std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H, 1ll << 40, 1).smem) > size_t(lim)) return false;
+    cudaError_t e = cudaSuccess;
+    for (auto k : {k_wgrad3<32>, k_wgrad3<16>, k_wgrad3<8>, k_wgrad3<4>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    for (auto k : {k_dgrad3<32>, k_dgrad3<16>, k_dgrad3<8>, k_dgrad3<4>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    return e == cudaSuccess;
 }
 
 }  // namespace net

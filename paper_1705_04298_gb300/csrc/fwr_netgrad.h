@@ -30,7 +30,7 @@ size_t wgrad_ws_floats(int cin, int cout, int H, int sms);
 // pixels that read each half-resolution one into lo [Bn][H/2][H/2][ca] (zeroed
 // where lo_act is not positive), the B part goes to dIn [Bn][H][H][cb].
 cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
-                       float* lo, const bf16* lo_act, cudaStream_t s);
+                       float* lo, const bf16* lo_act, int sms, cudaStream_t s);
 
 // Masked mean squared error of pred against T and the backward of the 1 x 1
 // output layer (C input channels a, two outputs): dIn [npix][C] (zeroed where
