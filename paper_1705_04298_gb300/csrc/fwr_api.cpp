@@ -312,7 +312,11 @@ fwr_status plan_create_n(fwr_plan** out, int n, int N, const uint8_t* pupil_mask
         } else {
             p->scratch_ctas = fwr::slab_max_ctas();
             const size_t b = size_t(p->scratch_ctas) * fwr::slab_scratch_elems_per_cta(N) * sizeof(float2);
-            if ((e = cudaMalloc(&p->d_scratch, b)) != cudaSuccess) st = cuda_fail(e, "cudaMalloc scratch");
+            const size_t cb = fwr::slab_counter_bytes(p->scratch_ctas);
+            if ((e = cudaMalloc(&p->d_scratch, b)) != cudaSuccess ||
+                (e = cudaMalloc(&p->d_counters, cb)) != cudaSuccess ||
+                (e = cudaMemset(p->d_counters, 0, cb)) != cudaSuccess)
+                st = cuda_fail(e, "cudaMalloc scratch");
             // the static array of fwr_reconstruct_static: its address on this
             // device, looked up now so that the allocation-free call itself
             // loads nothing; a failure here only disables that entry point
@@ -345,6 +349,7 @@ void fwr_plan_destroy(fwr_plan* p) {
     cudaFree(p->d_hud);
     cudaFree(p->d_status);
     cudaFree(p->d_scratch);
+    cudaFree(p->d_counters);
     cudaFree(p->d_dftws);
     cudaFree(p->d_stage_in);
     cudaFree(p->d_stage_out);
@@ -568,7 +573,7 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
         }
     } else if (p->N >= 256) {
         if (ext_out || !phase) return FWR_ERR_UNSUPPORTED;
-        e = fwr::launch_slab(p->N, k, p->d_scratch, p->scratch_ctas, static_cast<cudaStream_t>(stream));
+        e = fwr::launch_slab(p->N, k, p->d_scratch, p->d_counters, p->scratch_ctas, static_cast<cudaStream_t>(stream));
     } else {
         e = fwr::fused_supported(p->N, 4, p->n) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
                                                 : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
@@ -807,6 +812,9 @@ fwr_status fwr_get_status(fwr_plan* p) {
     unsigned v = 0;
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(&v, p->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost);
+    // a team barrier that gave up leaves its counters as they were
+    if (e == cudaSuccess && (v & fwr::STATUS_TIMEOUT) && p->d_counters)
+        e = cudaMemset(p->d_counters, 0, fwr::slab_counter_bytes(p->scratch_ctas));
     if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(unsigned));
     cudaSetDevice(prev);
     if (e != cudaSuccess) return cuda_fail(e, "status read");

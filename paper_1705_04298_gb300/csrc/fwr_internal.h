@@ -88,7 +88,12 @@ cudaError_t launch_dft2_gemm_f32(int N, const float2* in, float2* out, int F, in
 size_t slab_smem_bytes(int N, int n);
 size_t slab_scratch_elems_per_cta(int N);
 int slab_max_ctas();
-cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, int max_ctas, cudaStream_t s);
+// counters: slab_counter_bytes() of zeroed device memory that goes with the
+// scratch (team barriers; zero again after every launch).
+enum : int { TEAM_COUNTER_STRIDE = 32 };  // unsigneds per team: a 128-byte line each
+size_t slab_counter_bytes(int max_ctas);
+cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, unsigned* counters, int max_ctas,
+                        cudaStream_t s);
 // The same kernel on the library's static scratch array (no allocation):
 // at most STATIC_SLAB_GRIDS CTAs; cudaErrorInvalidValue for ctas outside
 // 1..STATIC_SLAB_GRIDS. static_slab_prepare (current device) returns the

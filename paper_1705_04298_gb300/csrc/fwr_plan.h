@@ -68,6 +68,7 @@ struct fwr_plan {
     fwr::DevTables<double> f64;
     // 256^2 grids: per-CTA global scratch of the slab kernel
     float2* d_scratch = nullptr;
+    unsigned* d_counters = nullptr;  // team barriers of the slab kernel (go with d_scratch)
     // 256^2 grids: device address of the library's static scratch array on the
     // plan's device (looked up at plan creation; nullptr if that failed)
     float2* d_static_scratch = nullptr;

@@ -33,9 +33,38 @@ slab_kernel(Params<float> p, float2* scratch) {
     if (threadIdx.x == 0 && s_bad) atomicOr(p.status, STATUS_NONFINITE);
 }
 
+// Few frames: a team of CTAs per frame. One frame's phases have too little
+// arithmetic and too few bytes in flight for more than one SM's share, and the
+// other SMs idle; the exchange through L2 is the same whoever does the slabs.
+// The grid is whole teams, all resident (a cooperative launch); bitwise the
+// results of slab_kernel (each line's and each bin's arithmetic is the same).
+// After a barrier's wait ran out (STATUS_TIMEOUT) the plan's team launches do
+// nothing until the status has been read, which also resets the counters.
+template <int N>
+__global__ void __launch_bounds__(SNT, 1)
+slab_team_kernel(Params<float> p, float2* scratch, unsigned* counters, int team) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (*reinterpret_cast<volatile unsigned*>(p.status) & STATUS_TIMEOUT) return;
+    SlabCtx c;
+    slab_setup<N>(c, smem, p.tab, p.mask, p.n, p.off, p.periodic);
+    const int teams = int(gridDim.x) / team, id = int(blockIdx.x) % teams, rank = int(blockIdx.x) / teams;
+    float2* G = scratch + size_t(id) * N * N;
+    TeamBar bar{counters + id * TEAM_COUNTER_STRIDE, 0u, team, false};
+    const int nn = p.n * p.n;
+    bool finite = true;
+    for (int f = id; f < p.F && !bar.dead; f += teams)
+        finite &= slab_frame<N, 2, true>(c, p.tab, p.slopes + size_t(f) * 2 * nn,
+                                         p.ext_init ? p.ext_init + size_t(f) * 2 * N * N : nullptr,
+                                         p.phase + size_t(f) * N * N, p.iters, G, p.hud, rank, &bar);
+    if (!bar.dead) team_leave(bar);
+    if (!finite) atomicOr(p.status, STATUS_NONFINITE);
+    if (bar.dead && threadIdx.x == 0) atomicOr(p.status, STATUS_TIMEOUT);
+}
+
 namespace {
 
 typedef void (*SlabKernel)(Params<float>, float2*);
+typedef void (*SlabTeamKernel)(Params<float>, float2*, unsigned*, int);
 
 // the kernel of grid N and a shape (1 or 2 warp groups; 0 is 2) with its
 // shared-memory limit set for n lenslets
@@ -51,6 +80,8 @@ size_t slab_smem_bytes(int N, int n) { return slab_layout_bytes_n(N, n); }
 
 size_t slab_scratch_elems_per_cta(int N) { return size_t(N) * N; }
 
+size_t slab_counter_bytes(int max_ctas) { return size_t(max_ctas) * TEAM_COUNTER_STRIDE * sizeof(unsigned); }
+
 int slab_max_ctas() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -58,8 +89,73 @@ int slab_max_ctas() {
     return sms;
 }
 
-cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, int max_ctas, cudaStream_t s) {
+namespace {
+
+// CTAs per frame. Cost of one wave of teams that fills the SMs (us, 128 x 128
+// on 256^2 and 200 x 200 on 512^2 lenslets, five iterations, 152 SMs; 1 is
+// slab_kernel; 8 and 32 slabs, two per CTA and step): a wave takes the same
+// time with fewer frames, so the least number of waves times their cost wins. At 512^2 teams of 8 also win for
+// many frames: 19 grids of 2 MB in flight stay in L2, 152 do not. Measured
+// with / without teams: 256^2, F = 1: 160 / 478, F = 38: 173 / 492, F = 200:
+// 846 / 1043; 512^2, F = 1: 194 / 2241, F = 16: 340 / 2320, F = 76: 1353 / 2746,
+// F = 152: 2707 / 2911.
+int team_size(int N, int F, int ctas) {
+    struct Cost {
+        int team, us;
+    };
+    static const Cost c256[] = {{1, 500}, {2, 286}, {4, 171}};
+    static const Cost c512[] = {{1, 2911}, {2, 1473}, {3, 990}, {4, 708}, {6, 485}, {8, 341}, {16, 197}};
+    const Cost* c = N == 512 ? c512 : c256;
+    const int nc = N == 512 ? 7 : 3;
+    int best = 1;
+    long long least = 0;
+    for (int i = 0; i < nc; ++i) {
+        const int teams = ctas / c[i].team;
+        if (teams < 1) continue;
+        const long long us = (long long)((F + teams - 1) / teams) * c[i].us;
+        if (i == 0 || us < least) {
+            least = us;
+            best = c[i].team;
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_team(int N, int team, const Params<float>& p, float2* scratch, unsigned* counters, int max_ctas,
+                        cudaStream_t s) {
+    const SlabTeamKernel kern = N == 512 ? slab_team_kernel<512> : slab_team_kernel<256>;
+    const size_t smem = slab_smem_bytes(N, p.n);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    int teams = max_ctas / team;
+    if (p.F < teams) teams = p.F;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(teams * team));
+    cfg.blockDim = dim3(SNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p, scratch, counters, team);
+}
+
+}  // namespace
+
+cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, unsigned* counters, int max_ctas,
+                        cudaStream_t s) {
     if (N != 256 && N != 512) return cudaErrorInvalidValue;
+    if (p.ctas == 0 && p.l2_bytes == 0 && p.shape != 1) {
+        const int team = team_size(N, p.F, max_ctas);
+        if (team > 1) {
+            cudaError_t e = launch_team(N, team, p, scratch, counters, max_ctas, s);
+            // fewer SMs to this context than the device has: one CTA per frame
+            if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+            cudaGetLastError();
+        }
+    }
     SlabKernel kern = nullptr;
     cudaError_t e = slab_kernel_for(N, p.shape, p.n, &kern);
     if (e != cudaSuccess) return e;

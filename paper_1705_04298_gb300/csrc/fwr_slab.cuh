@@ -107,6 +107,44 @@ __device__ __forceinline__ void group_sync(int g, int threads) {
     asm volatile("bar.sync %0, %1;\n" ::"r"(g + 1), "r"(threads) : "memory");
 }
 
+// Barrier of the CTAs that share a frame (all resident: a cooperative launch):
+// `count` is a counter in global memory that each CTA raises once per barrier,
+// and that team_leave returns to zero. The wait is bounded: after about two
+// seconds the CTA gives up and every thread gets false.
+struct TeamBar {
+    unsigned* count;   // [0]: arrivals, [1]: CTAs done (nullptr: no team)
+    unsigned target;   // arrivals that complete the next barrier
+    int team;
+    bool dead;         // a wait ran out
+};
+constexpr long long TEAM_WAIT = 4000000000ll;  // clock cycles
+
+__device__ __forceinline__ bool team_sync(TeamBar& b) {
+    __syncthreads();
+    bool ok = true;
+    b.target += b.team;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(b.count, 1u);
+        const long long t0 = clock64();
+        unsigned v;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(b.count) : "memory");
+            ok = v >= b.target;
+        } while (!ok && clock64() - t0 < TEAM_WAIT);
+        __threadfence();
+    }
+    b.dead = !__syncthreads_and(ok);
+    return !b.dead;
+}
+// after a CTA's last barrier: the last CTA of the team to come zeroes the counters
+__device__ __forceinline__ void team_leave(const TeamBar& b) {
+    if (threadIdx.x == 0 && atomicAdd(b.count + 1, 1u) == unsigned(b.team - 1)) {
+        b.count[0] = 0;
+        b.count[1] = 0;
+    }
+}
+
 // asynchronous global -> shared copies (cp.async), completed by cp_wait_all
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
@@ -211,8 +249,10 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
 }
 
 // One frame through the whole path with the grid in G (this CTA's N^2
-// scratch area). sl: [2][n][n] slopes; ext: [2][N][N] warm start or nullptr;
-// phase: [N][N] output. Called by every thread; returns false in the threads
+// scratch area). TEAM: the bar.team CTAs share the frame and G; CTA `rank`
+// takes every team-th pair of slabs and a team barrier ends each phase (a
+// frame whose barrier gave up is left unfinished, bar.dead set). sl:
+// [2][n][n] slopes; ext: [2][N][N] warm start or nullptr; phase: [N][N] output. Called by every thread; returns false in the threads
 // that saw a non-finite measured slope.
 //
 // Tasks (t: the thread's index in its group, i: its task): column phase,
@@ -221,14 +261,16 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
 // t / RB + (SGT / RB) i, RB-cell tasks (inverse pass A, forward pass B) index
 // t mod 16 and line t / 16 + (SGT / 16) i. Both shapes give bitwise the same
 // result (each line transform and each bin's arithmetic is the same).
-template <int N, int GROUPS>
+template <int N, int GROUPS, bool TEAM = false>
 __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>& tab, const float* sl,
                                            const float* ext, float* phase, int iters, float2* G,
-                                           const int16_t* hud = nullptr) {
+                                           const int16_t* hud = nullptr, int rank = 0, TeamBar* bar = nullptr) {
     typedef SlabShape<N, GROUPS> Sh;
     constexpr int SL = Sh::SL, SGT = Sh::SGT, SC = Sh::SC, WS = Sh::WS, RB = Sh::RB, H = Sh::H;
     constexpr int CLS = Sh::CLS, RLS_I = Sh::RLS_I, RLS_F = Sh::RLS_F, NA = Sh::NA, NB = Sh::NB;
     const int g = threadIdx.x / SGT, tg = threadIdx.x % SGT;
+    // first slab and step of this group
+    const int s0 = TEAM ? GROUPS * rank + g : g, ds = TEAM ? GROUPS * bar->team : GROUPS;
     float2* const Lb = c.Lb + g * Sh::LB_CELLS;
     const float2* const tw = c.tw;
     const float2* const twa = c.twa;
@@ -255,7 +297,7 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
         if (it >= 0) {
             // ------------------------------------------------ column phase
             const bool fill = mode == PERIODIC_BEFORE_EACH_FFT || (mode == PERIODIC_FINAL_ONLY && final);
-            for (int s = g; s < N / SL; s += GROUPS) {
+            for (int s = s0; s < N / SL; s += ds) {
                 const int kx = slab_col<N, SC>(s, cl);
                 const int pl = partner_line<SC>(s, cl);
                 {
@@ -383,12 +425,16 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                 group_sync(g, SGT);
             }
             // both groups' columns are in memory before any row is read
-            __syncthreads();
+            if (TEAM) {
+                if (!team_sync(*bar)) return finite;
+            } else {
+                __syncthreads();
+            }
         }
         // --------------------------------------------------------- row phase
         const bool fill_next = !final && (mode == PERIODIC_BEFORE_EACH_FFT ||
                                           (mode == PERIODIC_FINAL_ONLY && it + 1 == iters));
-        for (int b = g; b < N / SL; b += GROUPS) {
+        for (int b = s0; b < N / SL; b += ds) {
             const int m0 = SL * b;
             {
                 // this slab's measured slopes into L2 while it is loaded and transformed
@@ -528,7 +574,11 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
             group_sync(g, SGT);
         }
         // both groups' rows are in memory before the next column phase (or the next frame)
-        __syncthreads();
+        if (TEAM) {
+            if (!team_sync(*bar)) return finite;
+        } else {
+            __syncthreads();
+        }
     }
     return finite;
 }
