@@ -18,8 +18,9 @@
 // activations in FP32. The forward 3 x 3 convolutions whose input channel
 // groups are multiples of 16 (and output channels of 8) run on the tensor
 // cores as implicit GEMMs (mma.sync m16n8k16, BF16 in, FP32 accumulate); the
-// first and last layers, the backward pass and the small elementwise kernels
-// are SIMT.
+// first and last layers and the small elementwise kernels are SIMT. The
+// backward pass is in fwr_netgrad.cu; at width 16 the whole forward is one
+// kernel (fwr_netfwd.cu).
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -32,14 +33,12 @@
 
 #include "../../include/fwr.h"
 #include "fwr_internal.h"
+#include "fwr_netfwd.h"
 #include "fwr_netgrad.h"
 #include "fwr_plan.h"
 
 namespace fwr {
 namespace net {
-
-constexpr float IN_SCALE = 0.5f;
-constexpr int GRID = 128, LOW = 32, POOL = 4;
 
 // ----------------------------------------------------------------- kernels --
 
@@ -544,6 +543,41 @@ cudaError_t backward(fwr_net* n, int Bn, cudaStream_t s) {
     return conv_bwd(n, 0, g[0], n->X, nullptr, Bn, nullptr, nullptr, nullptr, nullptr, s);
 }
 
+// The whole forward in one kernel, where the width has it and the convolutions
+// are not forced to the CUDA cores: X, the activations and pools are kept for
+// the backward pass when `keep`, the prediction written as n->pred (keep) or
+// as the warm start ext.
+bool fused_forward(const fwr_net* n) {
+    if (n->w != FUSED_WIDTH || n->conv != FWR_NET_CONV_AUTO) return false;
+    for (int i = 1; i < 14; ++i)
+        if (!n->layers[i].tc) return false;
+    return true;
+}
+
+cudaError_t forward_fused(fwr_net* n, const fwr_plan* p, const float* slopes, int F, bool keep, float* ext,
+                          cudaStream_t s) {
+    FwdArgs a = {};
+    a.slopes = slopes;
+    a.mask = p->d_mask;
+    a.n = p->n;
+    a.off = p->off;
+    a.F = F;
+    a.w_first = n->Wb + n->layers[0].woff;
+    a.w_out = n->Wb + n->layers[14].woff;
+    for (int i = 0; i < 15; ++i) a.bias[i] = n->W + n->layers[i].boff;
+    for (int i = 1; i < 14; ++i) a.wp[i] = n->Wp + n->layers[i].poff;
+    a.ext = ext;
+    if (keep) {
+        a.pred = n->pred;
+        a.X = n->X;
+        for (int i = 0; i < 14; ++i) a.act[i] = n->act[i];
+        a.pool[0] = n->pool1;
+        a.pool[1] = n->pool2;
+        a.pool[2] = n->pool3;
+    }
+    return unet_forward(a, n->sms, s);
+}
+
 void free_net(fwr_net* n) {
     cudaFree(n->W);
     cudaFree(n->Wb);
@@ -663,6 +697,7 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
     }
+    if (e == cudaSuccess) e = unet_forward_prepare();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_conv_fwd<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fwd_smem));
     if (e != cudaSuccess) {
@@ -717,6 +752,11 @@ fwr_status fwr_net_forward(fwr_net* n, const fwr_plan* p, const float* slopes, i
     if (!n || !geometry_ok(p) || F < 0 || F > n->max_batch || (F > 0 && (!slopes || !ext_init))) return FWR_ERR_ARG;
     if (F == 0) return FWR_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // the kernel's warm-start rows are 16-byte stores
+    if (fused_forward(n) && (reinterpret_cast<uintptr_t>(ext_init) & 15u) == 0) {
+        const cudaError_t e = forward_fused(n, p, slopes, F, false, ext_init, s);
+        return e == cudaSuccess ? FWR_OK : fwr::cuda_fail(e, "fwr_net_forward");
+    }
     cudaError_t e = prepare(n, p, slopes, F, s);
     if (e == cudaSuccess) e = forward(n, F, s);
     if (e == cudaSuccess) {
@@ -732,14 +772,15 @@ fwr_status fwr_net_gradients(fwr_net* n, const fwr_plan* p, const float* slopes,
                              float* grad_host, float* loss_host, void* stream) {
     if (!n || !geometry_ok(p) || F < 1 || F > n->max_batch || !slopes || !target_ext) return FWR_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = prepare(n, p, slopes, F, s);
+    const bool fused = fused_forward(n);
+    cudaError_t e = fused ? forward_fused(n, p, slopes, F, true, nullptr, s) : prepare(n, p, slopes, F, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->cnt, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
         k_target<<<blocks(size_t(F) * LOW * LOW, 256), 256, 0, s>>>(target_ext, p->d_mask, p->n, p->off, F, n->T,
                                                                      n->LM, n->cnt);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = forward(n, F, s);
+    if (e == cudaSuccess && !fused) e = forward(n, F, s);
     if (e == cudaSuccess) e = backward(n, F, s);
     if (e == cudaSuccess && loss_host) e = cudaMemcpyAsync(loss_host, n->loss, sizeof(float), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && grad_host)
