@@ -15,7 +15,7 @@
 // epilogue's stores hit all banks; taps outside the image read a zero chunk.
 // 256 threads; the lifetimes are packed into 106 KB, so two CTAs share an SM
 // and one's barriers and epilogues overlap the other's products.
-// Measured, 1000 images and the warm start written: 1040 us layer by layer, 370 us.
+// Measured, 1000 images and the warm start written: 1040 us layer by layer, 320 us.
 
 #include "fwr_netfwd.h"
 
@@ -29,17 +29,20 @@ namespace {
 constexpr int NT = 256;
 constexpr int KB = 1024;
 // byte offsets of the activations (see the order of the layers in the kernel)
-constexpr int R0 = 0, R1 = 32 * KB, S2 = 64 * KB, S3 = 80 * KB, A11 = 88 * KB, ZERO = 104 * KB, WF = ZERO + 16,
+constexpr int R0 = 0, R1 = 32 * KB, S2 = 64 * KB, S3 = 80 * KB, A11 = 88 * KB, ZERO = 104 * KB, WF = ZERO + 128,
               WO = WF + 27 * 16 * 4, BF = WO + 32 * 4, SMEM = BF + 32 * 4;
 constexpr int P1 = R0, A2 = R0 + 8 * KB, P2 = R0, A4 = R0 + 4 * KB, P3 = R0 + 24 * KB, A6 = R0 + 26 * KB,
               A7 = R0 + 28 * KB, A8 = R0, A9 = R0 + 8 * KB, A10 = R0 + 16 * KB, A12 = R0, A13 = R1;
 static_assert(34 * 34 * 3 * 4 <= 16 * KB, "the input plane fits the space of layer 11's output");
 
-// byte offset of 16-byte chunk c of pixel p, C channels per pixel
+// permutation of a pixel's 16-byte chunks (2, 4 or 8 of them: C channels)
+template <int C> __device__ __forceinline__ int perm(int p) {
+    constexpr int n = C / 8;
+    return n == 2 ? (p >> 2) & 1 : n == 4 ? (p >> 1) & 3 : p & 7;
+}
+// byte offset of chunk c of pixel p
 template <int C> __device__ __forceinline__ uint32_t chunk_at(int p, int c) {
-    constexpr int n = C / 8;  // chunks per pixel (2, 4 or 8)
-    const int s = n == 2 ? (p >> 2) & 1 : n == 4 ? (p >> 1) & 3 : p & 7;
-    return uint32_t(p * C * 2 + ((c ^ s) << 4));
+    return uint32_t(p * C * 2 + ((c ^ perm<C>(p)) << 4));
 }
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&a)[4], uint32_t addr) {
@@ -57,46 +60,61 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
 
 // One 3 x 3 layer at H x H: input channels [A (CA, at half resolution when UP) |
 // B (CB)], COUT outputs, ReLU. WN warps across the output channels, 8 / WN across
-// the pixels. src*, dst: byte offsets of the activations in shared memory.
+// the pixels. src*, dst: byte offsets of the activations in shared memory. Starts
+// with the barrier that completes its input.
 template <int H, int CA, bool UP, int CB, int COUT, int WN>
 __device__ __forceinline__ void conv(unsigned char* sm, int srcA, int srcB, int dst, const uint2* __restrict__ wp,
                                      const float* __restrict__ bias, bf16* __restrict__ save) {
     constexpr int WM = 8 / WN, MTT = H * H / 16, NTT = COUT / 8, CH = (CA + CB) / 16;
-    constexpr int MT = MTT >= WM ? MTT / WM : 1, NTW = NTT / WN;
+    constexpr int MT = MTT / WM, NTW = NTT / WN;
+    static_assert(MT * WM == MTT && NTW * WN == NTT, "warps cover the layer");
+    // taps whose weights are loaded together, where the registers allow it (they
+    // come from L2: 1000 images 370 us a tap at a time, 320 with this and without
+    // a second warp on the same pixels at 16 x 16)
+    constexpr int TG = 3 * CH * NTW * 2 + MT * NTW * 4 <= 100 ? 3 : 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wm = warp / WN, wn = warp % WN;
-    if (MTT >= WM || wm < MTT) {
+    const uint2* w = wp + (wn * NTW) * 32 + lane;
+    __syncthreads();
+    {
         const uint32_t base = uint32_t(__cvta_generic_to_shared(sm));
         const int kh = lane >> 4;  // which 16-byte half of a 16-channel chunk
+        const int p0 = wm * MT * 16 + (lane & 15);
         float acc[MT][NTW][4];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
 #pragma unroll
             for (int t = 0; t < NTW; ++t) acc[m][t][0] = acc[m][t][1] = acc[m][t][2] = acc[m][t][3] = 0.f;
-        const uint2* w = wp + (wn * NTW) * 32 + lane;
 #pragma unroll 1
-        for (int tap = 0; tap < 9; ++tap) {
-            const int dy = tap / 3 - 1, dx = tap - (tap / 3) * 3 - 1;
-            uint2 b[CH][NTW];
+        for (int t0 = 0; t0 < 9; t0 += TG) {
+            uint2 b[TG][CH][NTW];
 #pragma unroll
-            for (int c = 0; c < CH; ++c)
+            for (int i = 0; i < TG * CH; ++i)
 #pragma unroll
-                for (int t = 0; t < NTW; ++t) b[c][t] = __ldg(w + (c * NTT + t) * 32);
-            w += CH * NTT * 32;
+                for (int t = 0; t < NTW; ++t) b[i / CH][i % CH][t] = __ldg(w + (i * NTT + t) * 32);
+            w += TG * CH * NTT * 32;
 #pragma unroll
-            for (int m = 0; m < MT; ++m) {
-                const int p = (wm * MT + m) * 16 + (lane & 15), y = p / H + dy, x = p % H + dx;
-                const bool in = y >= 0 && y < H && x >= 0 && x < H;
-                const int pa = UP ? (y >> 1) * (H / 2) + (x >> 1) : y * H + x, pb = y * H + x;
+            for (int g = 0; g < TG; ++g) {
+                const int dy = t0 / 3 - 1, dx = TG == 3 ? g - 1 : t0 - (t0 / 3) * 3 - 1;
+                // this lane's pixel of tile m is p0 + 16 m; a tap's chunk permutation
+                // is the same for all tiles where the rows hold whole tiles' low bits
+                const int x0 = p0 % H + dx, y0 = p0 / H + dy;
 #pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    uint32_t off;
-                    if (16 * c < CA) off = uint32_t(srcA) + chunk_at<CA>(pa, 2 * c + kh);
-                    else off = uint32_t(srcB) + chunk_at<CB ? CB : 16>(pb, 2 * c - CA / 8 + kh);
-                    uint32_t a[4];
-                    ldsm_x4(a, base + (in ? off : uint32_t(ZERO)));
+                for (int m = 0; m < MT; ++m) {
+                    const int x = x0 + (16 * m) % H, y = y0 + (16 * m) / H;
+                    const bool in = y >= 0 && y < H && x >= 0 && x < H;
+                    const int pa = UP ? (y >> 1) * (H / 2) + (x >> 1) : y * H + x, pb = y * H + x;
+                    const uint32_t am = base + (in ? uint32_t(srcA + pa * CA * 2) : uint32_t(ZERO));
+                    const uint32_t bm = base + (in ? uint32_t(srcB + pb * CB * 2) : uint32_t(ZERO));
+                    const int sa = perm<CA>(pa), sb = perm<CB ? CB : 16>(pb);
 #pragma unroll
-                    for (int t = 0; t < NTW; ++t) mma_16816(acc[m][t], a, b[c][t]);
+                    for (int c = 0; c < CH; ++c) {
+                        uint32_t a[4];
+                        if (16 * c < CA) ldsm_x4(a, am + (((2 * c + kh) ^ sa) << 4));
+                        else ldsm_x4(a, bm + (((2 * c - CA / 8 + kh) ^ sb) << 4));
+#pragma unroll
+                        for (int t = 0; t < NTW; ++t) mma_16816(acc[m][t], a, b[g][c][t]);
+                    }
                 }
             }
         }
@@ -117,13 +135,13 @@ __device__ __forceinline__ void conv(unsigned char* sm, int srcA, int srcB, int 
                 }
         }
     }
-    __syncthreads();
 }
 
-// 2 x 2 average pooling of an H x H x C activation
+// 2 x 2 average pooling of an H x H x C activation; starts with a barrier
 template <int H, int C>
 __device__ __forceinline__ void pool(unsigned char* sm, int src, int dst, bf16* __restrict__ save) {
     constexpr int Ho = H / 2;
+    __syncthreads();
     for (int i = threadIdx.x; i < Ho * Ho * (C / 8); i += NT) {
         const int c = i % (C / 8), p = i / (C / 8), y = p / Ho, x = p % Ho;
         float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -145,7 +163,6 @@ __device__ __forceinline__ void pool(unsigned char* sm, int src, int dst, bf16* 
         *reinterpret_cast<uint4*>(sm + dst + chunk_at<C>(p, c)) = v;
         if (save) *reinterpret_cast<uint4*>(save + size_t(p) * C + 8 * c) = v;
     }
-    __syncthreads();
 }
 
 __global__ void __launch_bounds__(NT, 2) k_unet_forward(const __grid_constant__ FwdArgs a) {
@@ -159,7 +176,7 @@ __global__ void __launch_bounds__(NT, 2) k_unet_forward(const __grid_constant__ 
     if (tid < 32) wo[tid] = __bfloat162float(a.w_out[tid]);
     if (tid < 16) bf[tid] = a.bias[0][tid];
     if (tid < 2) bf[16 + tid] = a.bias[14][tid];
-    if (tid < 4) reinterpret_cast<uint32_t*>(sm + ZERO)[tid] = 0u;
+    if (tid < 32) reinterpret_cast<uint32_t*>(sm + ZERO)[tid] = 0u;
     const int n = a.n, nn = n * n;
     for (int f = blockIdx.x; f < a.F; f += gridDim.x) {
         auto at = [&](bf16* p, int per) { return p ? p + size_t(f) * per : nullptr; };
@@ -247,11 +264,10 @@ __global__ void __launch_bounds__(NT, 2) k_unet_forward(const __grid_constant__ 
                 }
             }
         }
-        __syncthreads();
         conv<32, 16, false, 0, 16, 1>(sm, R0, 0, R1, a.wp[1], a.bias[1], at(a.act[1], 1024 * 16));
         pool<32, 16>(sm, R1, P1, at(a.pool[0], 256 * 16));
-        conv<16, 16, false, 0, 32, 2>(sm, P1, 0, A2, a.wp[2], a.bias[2], at(a.act[2], 256 * 32));
-        conv<16, 32, false, 0, 32, 2>(sm, A2, 0, S2, a.wp[3], a.bias[3], at(a.act[3], 256 * 32));
+        conv<16, 16, false, 0, 32, 1>(sm, P1, 0, A2, a.wp[2], a.bias[2], at(a.act[2], 256 * 32));
+        conv<16, 32, false, 0, 32, 1>(sm, A2, 0, S2, a.wp[3], a.bias[3], at(a.act[3], 256 * 32));
         pool<16, 32>(sm, S2, P2, at(a.pool[1], 64 * 32));
         conv<8, 32, false, 0, 64, 4>(sm, P2, 0, A4, a.wp[4], a.bias[4], at(a.act[4], 64 * 64));
         conv<8, 64, false, 0, 64, 4>(sm, A4, 0, S3, a.wp[5], a.bias[5], at(a.act[5], 64 * 64));
@@ -260,11 +276,12 @@ __global__ void __launch_bounds__(NT, 2) k_unet_forward(const __grid_constant__ 
         conv<4, 64, false, 0, 64, 8>(sm, A6, 0, A7, a.wp[7], a.bias[7], at(a.act[7], 16 * 64));
         conv<8, 64, true, 64, 64, 4>(sm, A7, S3, A8, a.wp[8], a.bias[8], at(a.act[8], 64 * 64));
         conv<8, 64, false, 0, 64, 4>(sm, A8, 0, A9, a.wp[9], a.bias[9], at(a.act[9], 64 * 64));
-        conv<16, 64, true, 32, 32, 2>(sm, A9, S2, A10, a.wp[10], a.bias[10], at(a.act[10], 256 * 32));
-        conv<16, 32, false, 0, 32, 2>(sm, A10, 0, A11, a.wp[11], a.bias[11], at(a.act[11], 256 * 32));
+        conv<16, 64, true, 32, 32, 1>(sm, A9, S2, A10, a.wp[10], a.bias[10], at(a.act[10], 256 * 32));
+        conv<16, 32, false, 0, 32, 1>(sm, A10, 0, A11, a.wp[11], a.bias[11], at(a.act[11], 256 * 32));
         conv<32, 32, true, 16, 16, 1>(sm, A11, R1, A12, a.wp[12], a.bias[12], at(a.act[12], 1024 * 16));
         conv<32, 16, false, 0, 16, 1>(sm, A12, 0, A13, a.wp[13], a.bias[13], at(a.act[13], 1024 * 16));
         // output layer; the warm start repeats it over 4 x 4 blocks
+        __syncthreads();
         for (int p = tid; p < LOW * LOW; p += NT) {
             const uint4 c0 = *reinterpret_cast<const uint4*>(sm + A13 + chunk_at<16>(p, 0));
             const uint4 c1 = *reinterpret_cast<const uint4*>(sm + A13 + chunk_at<16>(p, 1));

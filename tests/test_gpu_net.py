@@ -156,3 +156,20 @@ def test_gradients_at_other_widths(fwr, w, F):
     assert abs(loss - loss_o) <= 2e-2 * abs(loss_o)
     rel = np.linalg.norm(g - g_o) / np.linalg.norm(g_o)
     assert rel <= 5e-2, rel
+
+
+@pytest.mark.parametrize("n,F", [(40, 1), (37, 5), (64, 307)])
+def test_one_kernel_forward_matches_layers(fwr, n, F):
+    """Width 16: the one-kernel forward (more images than it has CTAs in the
+    last case) gives bitwise the layered path's warm start, which serves an
+    output that is not 16-byte aligned."""
+    rng = np.random.default_rng(n)
+    plan = fwr.Plan(synth.pupil_mask(n), 1.0, fwr.LSQ, grid=128)
+    net = fwr.Net(16, F, unet.init_params(16, 3) + 0.02 * rng.standard_normal(unet.param_count(16)))
+    s = torch.randn((F, 2, n, n), device="cuda")
+    a = net.forward(plan, s)
+    buf = torch.empty(F * 2 * 128 * 128 + 1, device="cuda")
+    b = buf[1:].view(F, 2, 128, 128)
+    assert b.data_ptr() % 16 == 4
+    net.forward(plan, s, b)
+    assert torch.equal(a, b)
