@@ -273,9 +273,10 @@ fwr_status plan_create_n(fwr_plan** out, int n, int N, const uint8_t* pupil_mask
     p->L0 = L0;
     p->nvalid = nvalid;
     cudaError_t e = cudaGetDevice(&p->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) {
         delete p;
-        return cuda_fail(e, "cudaGetDevice");
+        return cuda_fail(e, "plan device");
     }
     std::vector<uint8_t> m(size_t(n) * n);
     for (int i = 0; i < n * n; ++i) m[i] = pupil_mask[i] ? 1 : 0;
@@ -666,6 +667,9 @@ fwr_status fwr_reconstruct_f64(fwr_plan* p, const double* slopes, const double* 
         k.hud = p->d_hud;
     }
     cudaError_t e = !pow2(p->N) ? fwr::launch_anygrid_f64(p->N, k, static_cast<cudaStream_t>(stream))
+                    // few frames on every SM (no FWR_OPT_CTAS)
+                    : phase && !ext_out && p->ctas == 0 && fwr::cluster64_wanted(p->N, n_frames, p->sms)
+                        ? fwr::launch_cluster_f64(p->N, k, static_cast<cudaStream_t>(stream))
                     : fwr::fused_supported(p->N, 8, p->n)
                         ? fwr::launch_fused_f64(p->N, k, static_cast<cudaStream_t>(stream))
                         : fwr::launch_basic_f64(p->N, k, static_cast<cudaStream_t>(stream));
@@ -682,10 +686,6 @@ fwr_status fwr_plan_reserve(fwr_plan* p, int n_frames) {
         for (cudaEvent_t* ev : {&p->ev_start, &p->ev_in, &p->ev_k, &p->ev_done})
             if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess)
                 return cuda_fail(e, "cudaEventCreate (host path)");
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-            (e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-            return cuda_fail(e, "device attributes (host path)");
     }
     if (n_frames <= p->stage_frames) return FWR_OK;
     cudaFree(p->d_stage_in);

@@ -139,6 +139,12 @@ bool fused_supported(int N, int elem_bytes, int n);
 cudaError_t launch_fused_f32(int N, const Params<float>& p, cudaStream_t s);
 cudaError_t launch_fused_f64(int N, const Params<double>& p, cudaStream_t s);
 
+// FP64 with a cluster of CTAs per frame (fwr_cluster64.cu), for few frames on
+// 32^2 and 64^2 grids; needs a phase output and has no ext_out.
+// cluster64_wanted: whether it is the faster one for F frames on `sms` SMs.
+bool cluster64_wanted(int N, int F, int sms);
+cudaError_t launch_cluster_f64(int N, const Params<double>& p, cudaStream_t s);
+
 // Standalone batched 2-D FFT (test entry), FP32.
 cudaError_t launch_fft2_f32(int N, const float2* in, float2* out, int F, int inverse,
                             const float2* tw, cudaStream_t s);
