@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "fwr_internal.h"
@@ -40,19 +41,12 @@ namespace fwr {
 
 #include "fwr_fft.cuh"
 #include "fwr_fused.cuh"
+#include "fwr_cluster.cuh"
 
 namespace {
 
 constexpr int CL = 8;  // CTAs per frame
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
-// store v at this CTA's shared-memory address a in CTA `rank` of the cluster
-__device__ __forceinline__ void st_rank(uint32_t a, int rank, double2 v) {
-    uint32_t o;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(o) : "r"(a), "r"(rank));
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};\n" ::"r"(o), "d"(v.x), "d"(v.y) : "memory");
-}
 __device__ __forceinline__ double2 shfl_xor2(double2 v, int h) {
     return make_double2(__shfl_xor_sync(0xffffffffu, v.x, h), __shfl_xor_sync(0xffffffffu, v.y, h));
 }
@@ -63,16 +57,6 @@ template <int N> struct C64 {
     static constexpr size_t rbuf = 0, cbuf = rbuf + size_t(SL) * LS * 16, sbuf = cbuf + size_t(SL) * LS * 16,
                             dc = sbuf + size_t(SL) * LS * 16, bytes = dc + size_t(SL) * 16;
 };
-
-// Eq. 2 on one bin: phi = Rx Sx + Ry Sy with 2 Sx = z1 + conj z2, 2 Sy = (z1 -
-// conj z2) / i; w = half the final weight
-__device__ __forceinline__ double2 final_bin(double2 z1, double2 z2, double2 Akx, double2 Tkx, double2 Aky, double2 Tky,
-                                             double w) {
-    const double2 sx = make_double2(z1.x + z2.x, z1.y - z2.y), sy = make_double2(z1.y + z2.y, z2.x - z1.x);
-    const double2 gx = cmul(Akx, Tky), gy = cmul(Tkx, Aky);
-    const double2 ph = cadd(cmulc(gx, sx), cmulc(gy, sy));
-    return make_double2(ph.x * w, ph.y * w);
-}
 
 // this lane's constants: signs of the trivial stages, +-w_8^J and +-w_16^J of
 // the others (J: the pair's place in its block), the twiddles w_N^(n2 k1) of its
@@ -150,9 +134,7 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
     double2* const dc = reinterpret_cast<double2*>(smem + G::dc);   // [line] column sums
     const uint32_t rbase = uint32_t(__cvta_generic_to_shared(R)), cbase = uint32_t(__cvta_generic_to_shared(C));
     const int lane = threadIdx.x & 31, line = threadIdx.x >> 5;
-    uint32_t rk;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rk));
-    const int rank = int(rk), n = p.n, off = p.off, nn = n * n, mode = p.periodic;
+    const int rank = cluster_rank(), n = p.n, off = p.off, nn = n * n, mode = p.periodic;
     cluster_arrive();  // matched before the first remote store: every CTA runs
 
     Tw64<N> tw;
@@ -176,10 +158,8 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
             tw.t[e] = p.tab.tw[n2 * (j % (N / 4))];
         }
     }
-    // column: kx of this warp's line (SC first-half columns, their partners, the
-    // self-paired N/2 in place of the second 0), the line of -kx
-    const int jj = line - SC;
-    const int kx = line < SC ? SC * rank + line : (rank == 0 && jj == 0) ? H : (N - SC * rank - jj) & (N - 1);
+    // column of this warp's line, the line of its partner -kx
+    const int kx = owned_column<N, SC>(rank, line);
     const int kxn = (N - kx) & (N - 1);
     const int pl = (rank == 0 && (line & (SC - 1)) == 0) ? line : (line ^ SC);
     // this lane's elements j = lane + 32 e: bin (j, kx), row j of a column,
@@ -260,8 +240,8 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
             line_dft<false, N>(x, tw, lane);
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const int c = lane + 32 * e, k = c < H ? c : N - c;
-                const int owner = c == H ? 0 : k / SC, l = c == H ? SC : k % SC + (c < H ? 0 : SC);
+                int owner, l;
+                column_owner<N, SC>(lane + 32 * e, owner, l);
                 st_rank(cbase + uint32_t((l * LS + row) * 16), owner, x[e]);
             }
             cluster_arrive();
@@ -328,39 +308,9 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
 }
 
 template <int N> cudaError_t launch_n(const Params<double>& p, cudaStream_t s) {
-    typedef C64<N> G;
     static std::mutex mu;
-    static std::vector<std::pair<int, int>> resident;  // device, clusters
-    auto kern = cluster64_kernel<N>;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(G::NT);
-    cfg.dynamicSmemBytes = G::bytes;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int dev = 0, clusters = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        for (const auto& r : resident)
-            if (r.first == dev) clusters = r.second;
-        if (clusters == 0) {
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(G::bytes))) != cudaSuccess)
-                return e;
-            if ((e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg)) != cudaSuccess) return e;
-            if (clusters < 1) return cudaErrorInvalidConfiguration;
-            resident.push_back({dev, clusters});
-        }
-    }
-    if (p.F < clusters) clusters = p.F;
-    cfg.gridDim = dim3(CL * clusters);
-    return cudaLaunchKernelEx(&cfg, kern, p, clusters);
+    static std::vector<std::pair<int, int>> cache;
+    return launch_clusters(cluster64_kernel<N>, p, CL, C64<N>::NT, C64<N>::bytes, mu, cache, s);
 }
 
 }  // namespace

@@ -18,6 +18,18 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
 template <typename V> __device__ __forceinline__ V cmulc(V a, V b) {
     return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
+__device__ __forceinline__ float mulrn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mulrn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fmadd(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
+// a b and conj(a) b with every operation written out (which product is fused
+// is not left to the compiler): kernels that share them agree bitwise
+template <typename V> __device__ __forceinline__ V cmul_rn(V a, V b) {
+    return mk(fmadd(a.x, b.x, -mulrn(a.y, b.y)), fmadd(a.x, b.y, mulrn(a.y, b.x)));
+}
+template <typename V> __device__ __forceinline__ V cmulc_rn(V a, V b) {
+    return mk(fmadd(a.x, b.x, mulrn(a.y, b.y)), fmadd(a.x, b.y, -mulrn(a.y, b.x)));
+}
 template <int R> struct Log2 { static constexpr int v = 1 + Log2<R / 2>::v; };
 template <> struct Log2<1> { static constexpr int v = 0; };
 
@@ -27,8 +39,6 @@ __host__ __device__ constexpr int bitrev(int i, int bits) {
     return r;
 }
 
-__device__ __forceinline__ float fmadd(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fmadd(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float2 t32(float2, int i) { return c_t32f[i]; }
 __device__ __forceinline__ double2 t32(double2, int i) { return c_t32d[i]; }
 

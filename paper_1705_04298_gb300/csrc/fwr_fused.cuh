@@ -145,9 +145,6 @@ __device__ __forceinline__ quad<float> load_pt(const float* p) {
 }
 __device__ __forceinline__ quad<double> load_pt(const double* p) { return {p[0], p[1], p[2], p[3]}; }
 
-__device__ __forceinline__ float mulrn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mulrn(double a, double b) { return __dmul_rn(a, b); }
-
 // LSQ projection of one bin pair (Algorithm 1 step 2, formula of Sec. 3.3)
 // with the separable factors p(u) = a(u) conj T(u), |a(u)|^2, |T(u)|^2 of the
 // bin's column (pux, puy, 2 ha2u = |a(u)|^2, 2 ht2u = |T(u)|^2) and row (pv),
@@ -171,6 +168,33 @@ __device__ __forceinline__ void lsq_coefs(T w, T pux, T puy, T ha2u, T ht2u, con
 template <typename T, typename V>
 __device__ __forceinline__ V lsq_apply(T al, T be, T ga, V z1, V z2) {
     return mk(fmadd(al, z1.x, fmadd(be, z2.x, mulrn(ga, z2.y))), fmadd(al, z1.y, fmadd(ga, z2.x, -mulrn(be, z2.y))));
+}
+
+// Final filter of one bin (Eq. 2): phi = Rx Sx + Ry Sy with 2 Sx = z1 + conj
+// z2, 2 Sy = (z1 - conj z2) / i; w is half the final weight. Written out like
+// lsq_coefs.
+template <typename T, typename V>
+__device__ __forceinline__ V final_bin(V z1, V z2, V Akx, V Tkx, V Aky, V Tky, T w) {
+    const V z2c = mk(z2.x, -z2.y);
+    const V sx = cadd(z1, z2c);
+    const V dd = csub(z1, z2c);
+    const V sy = mk(dd.y, -dd.x);
+    const V gx = cmul_rn(Akx, Tky);
+    const V gy = cmul_rn(Tkx, Aky);
+    // conj(gx) sx + conj(gy) sy
+    const V ph = mk(fmadd(gx.x, sx.x, fmadd(gx.y, sx.y, fmadd(gy.x, sy.x, mulrn(gy.y, sy.y)))),
+                    fmadd(gx.x, sx.y, fmadd(-gx.y, sx.x, fmadd(gy.x, sy.y, -mulrn(gy.y, sy.x)))));
+    return mk(mulrn(ph.x, w), mulrn(ph.y, w));
+}
+// y part of Eq. PC: the last input of a column task's forward DFT with the
+// fill added, from the uncorrected ky = 0 bins of the column and its partner
+// and t = w_N^q1 of the task's first bin
+template <typename V>
+__device__ __forceinline__ V fill_input(V xlast, V z0, V z0p, V t) {
+    typedef decltype(V().x) T;
+    const V ey = mk(T(0.5) * (z0.y + z0p.y), T(0.5) * (z0p.x - z0.x));
+    const V c0 = cmul_rn(ey, mk(t.x, -t.y));
+    return mk(xlast.x + c0.y, xlast.y - c0.x);
 }
 
 // Tensor memory as per-thread storage (32x32b shape: a thread reaches the
@@ -200,7 +224,7 @@ constexpr uint32_t FUSED_TMEM_COLS = 512;
 
 template <bool INV, typename V>
 __device__ __forceinline__ V twiddle(V x, V w) {
-    return INV ? cmulc(w, x) : cmul(x, w);
+    return INV ? cmulc_rn(w, x) : cmul_rn(x, w);
 }
 
 // P2 in either direction over all R*R tasks (row radix-4 x column radix-4).
@@ -481,7 +505,6 @@ __device__ __forceinline__ bool fused_frame(const FusedCtx<T, N>& c, const T* sl
     const T* const ion = c.ion;
     const T* const wfp = c.wfp;
     const T* const wfn = c.wfn;
-    const T half = T(0.5);
     bool finite = true;
     const bool warm = ext || exth;
     if (warm) {
@@ -618,11 +641,7 @@ __device__ __forceinline__ bool fused_frame(const FusedCtx<T, N>& c, const T* sl
                 dc[gam] = t[0];
             }
             __syncthreads();
-            const V z0 = dc[gam], z0p = dc[gamp];
-            const V ey = mk(half * (z0.y + z0p.y), half * (z0p.x - z0.x));
-            const V tq = twv[0];
-            const V c0 = cmul(ey, mk(tq.x, -tq.y));
-            x[R - 1] = mk(x[R - 1].x + c0.y, x[R - 1].y - c0.x);
+            x[R - 1] = fill_input(x[R - 1], dc[gam], dc[gamp], twv[0]);
         }
         dft_reg<R, false>(x);
 #pragma unroll
@@ -666,20 +685,12 @@ __device__ __forceinline__ bool fused_frame(const FusedCtx<T, N>& c, const T* sl
             for (int q2 = 0; q2 < R; ++q2) {
                 const V z2 = q2 == 0 ? (q1 == 0 ? partp[0] : partp[S * (R - 1)]) : partq[S * (R - 1 - q2)];
                 const V z1 = x[q2];
-                const V z2c = mk(z2.x, -z2.y);
                 // ky = 4 q2 + q1 <= N/2: weight stored at (ky, kx); known at
                 // compile time except for q2 = N/8
                 const bool lo = q2 < R / 2 || (q2 == R / 2 && q1 == 0);
-                // Eq. 2: phi = Rx Sx + Ry Sy with 2 Sx = z1 + conj z2, 2 Sy = (z1 - conj z2) / i
                 const int ky = q1 + 4 * q2;
-                const V sx = cadd(z1, z2c);
-                const V dd = csub(z1, z2c);
-                const V sy = mk(dd.y, -dd.x);
-                const V gx = cmul(Ax, Tt[ky]);
-                const V gy = cmul(Tx, A[ky]);
-                const T w = half * (lo ? wfp[4 * N * q2] : wfn[-4 * N * q2]);
-                const V ph = cadd(cmulc(gx, sx), cmulc(gy, sy));
-                x[q2] = mk(ph.x * w, ph.y * w);
+                x[q2] = final_bin(z1, z2, Ax, Tx, A[ky], Tt[ky],
+                                  T(0.5) * (lo ? wfp[4 * N * q2] : wfn[-4 * N * q2]));
             }
         }
         // ---- P3 inverse

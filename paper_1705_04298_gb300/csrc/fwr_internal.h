@@ -139,6 +139,12 @@ bool fused_supported(int N, int elem_bytes, int n);
 cudaError_t launch_fused_f32(int N, const Params<float>& p, cudaStream_t s);
 cudaError_t launch_fused_f64(int N, const Params<double>& p, cudaStream_t s);
 
+// FP32, 128^2, with a cluster of CTAs per frame (fwr_cluster128.cu): bitwise the
+// fused kernel's phase; needs a phase output and has no ext_out.
+// cluster128_wanted: whether it is the faster one for F frames on `sms` SMs.
+bool cluster128_wanted(int F, int sms);
+cudaError_t launch_cluster_f32(const Params<float>& p, int sms, cudaStream_t s);
+
 // FP64 with a cluster of CTAs per frame (fwr_cluster64.cu), for few frames on
 // 32^2 and 64^2 grids; needs a phase output and has no ext_out.
 // cluster64_wanted: whether it is the faster one for F frames on `sms` SMs.
