@@ -67,10 +67,11 @@ template <int N, int GROUPS> struct SlabShape {
     static constexpr int SC = SL / 2;                       // first-half columns of a column slab
     static constexpr int WS = SC + 1;                       // row stride of a group's spectral weights
     static constexpr int CLS = N + 1;                       // column phase: line stride (cells)
-    static constexpr int RLS_I = RB * 17;                   // row phase, inverse: groups of 16, stride 17
-    static constexpr int RLS_F = 16 * (RB + 1);             // row phase, forward: groups of RB, stride RB + 1
-    static constexpr int M1 = SL * CLS > SL * RLS_I ? SL * CLS : SL * RLS_I;
-    static constexpr int LB_CELLS = M1 > SL * RLS_F ? M1 : SL * RLS_F;  // one group's buffer
+    // row phase: a line's groups of 16, stride 17 (inverse), or of RB, stride
+    // RB + 1 (forward), in the same cells
+    static constexpr int RLS = RB * 17;
+    static_assert(16 * (RB + 1) <= RLS, "both exchanges fit a line");
+    static constexpr int LB_CELLS = SL * CLS > SL * RLS ? SL * CLS : SL * RLS;  // one group's buffer
     static constexpr int NA = SL * RB / SGT;                // 16-point tasks per thread and pass
     static constexpr int NB = SL * 16 / SGT;                // RB-point tasks per thread and pass
     static_assert(NA * SGT == SL * RB && NB * SGT == SL * 16, "tasks divide evenly");
@@ -252,22 +253,27 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
 // scratch area). TEAM: the bar.team CTAs share the frame and G; CTA `rank`
 // takes every team-th pair of slabs and a team barrier ends each phase (a
 // frame whose barrier gave up is left unfinished, bar.dead set). sl:
-// [2][n][n] slopes; ext: [2][N][N] warm start or nullptr; phase: [N][N] output. Called by every thread; returns false in the threads
-// that saw a non-finite measured slope.
+// [2][n][n] slopes; ext: [2][N][N] warm start or nullptr; phase: [N][N]
+// output. Called by every thread; returns false in the threads that saw a
+// non-finite measured slope.
 //
 // Tasks (t: the thread's index in its group, i: its task): column phase,
 // line t mod SL and pass index q = t / SL + (SGT / SL) i; row phase, 16-cell
 // tasks (inverse pass B, forward pass A) take index t mod RB and line
-// t / RB + (SGT / RB) i, RB-cell tasks (inverse pass A, forward pass B) index
-// t mod 16 and line t / 16 + (SGT / 16) i. Both shapes give bitwise the same
-// result (each line transform and each bin's arithmetic is the same).
+// t / 16 + (SGT / 16) i at 256^2, 2 (t / 32) + i at 512^2, RB-cell tasks
+// (inverse pass A, forward pass B) index t mod 16 and line t / 16 + (SGT / 16) i:
+// all tasks of a row are in one warp, so the row phase's exchanges need no
+// barrier of the group and its warps run apart (1000 frames of 128 x 128
+// lenslets on 256^2, k = 10: 6.65 ms with a group barrier at each exchange,
+// 6.36 without). Both shapes give bitwise the same result (each line transform
+// and each bin's arithmetic is the same).
 template <int N, int GROUPS, bool TEAM = false>
 __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>& tab, const float* sl,
                                            const float* ext, float* phase, int iters, float2* G,
                                            const int16_t* hud = nullptr, int rank = 0, TeamBar* bar = nullptr) {
     typedef SlabShape<N, GROUPS> Sh;
     constexpr int SL = Sh::SL, SGT = Sh::SGT, SC = Sh::SC, WS = Sh::WS, RB = Sh::RB, H = Sh::H;
-    constexpr int CLS = Sh::CLS, RLS_I = Sh::RLS_I, RLS_F = Sh::RLS_F, NA = Sh::NA, NB = Sh::NB;
+    constexpr int CLS = Sh::CLS, RLS = Sh::RLS, NA = Sh::NA, NB = Sh::NB;
     const int g = threadIdx.x / SGT, tg = threadIdx.x % SGT;
     // first slab and step of this group
     const int s0 = TEAM ? GROUPS * rank + g : g, ds = TEAM ? GROUPS * bar->team : GROUPS;
@@ -287,8 +293,9 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
     constexpr int CQS = SGT / SL;
     // row-phase roles
     const int r16 = tg % 16, l16 = tg / 16;   // RB-cell tasks
-    const int rrb = tg % RB, lrb = tg / RB;   // 16-cell tasks
-    constexpr int L16S = SGT / 16, LRBS = SGT / RB;
+    constexpr int L16S = SGT / 16, LRBS = RB == 16 ? L16S : 1;
+    const int rrb = tg % RB, lrb = RB == 16 ? tg / 16 : NA * (tg / 32);   // 16-cell tasks
+    static_assert(RB == 16 || (NB == 1 && NA == 2), "a row's tasks in one warp");
     // the RB lanes of one row's 16-cell tasks (for the x-fill row sums)
     const unsigned row_mask = RB == 32 ? 0xFFFFFFFFu : (0xFFFFu << (threadIdx.x & 16));
     // it = -1: embed; it = 0 .. iters-1: Gerchberg; it = iters: final
@@ -324,6 +331,8 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                     for (int i = 0; i < NA; ++i) {
                         const int n2 = cq + CQS * i;
                         dft_tw<16, false>(x[i], twa + n2, RB);
+                        // the slab before: every inverse pass B has read its cells
+                        if (i == 0) group_sync(g, SGT);
 #pragma unroll
                         for (int k1 = 0; k1 < 16; ++k1) Lb[cl * CLS + RB * k1 + n2] = x[i][k1];
                     }
@@ -422,7 +431,6 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                         for (int k2 = 0; k2 < 16; ++k2) __stcg(G + (k1 + RB * k2) * N + kx, x[i][k2]);
                     }
                 }
-                group_sync(g, SGT);
             }
             // both groups' columns are in memory before any row is read
             if (TEAM) {
@@ -486,17 +494,18 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                     for (int i = 0; i < NB; ++i) {
                         const int line = l16 + L16S * i;
                         dft_tw<RB, true>(y[i], twi + r16, 16);
+                        if (i == 0) __syncwarp();  // the slab before: every forward pass B has read its cells
 #pragma unroll
-                        for (int k1 = 0; k1 < RB; ++k1) Lb[line * RLS_I + 17 * k1 + r16] = y[i][k1];
+                        for (int k1 = 0; k1 < RB; ++k1) Lb[line * RLS + 17 * k1 + r16] = y[i][k1];
                     }
                 }
-                group_sync(g, SGT);
+                __syncwarp();
                 // inverse pass B: cells rrb + RB k2 of the row
 #pragma unroll
                 for (int i = 0; i < NA; ++i) {
                     const int line = lrb + LRBS * i;
 #pragma unroll
-                    for (int n2 = 0; n2 < 16; ++n2) x[i][n2] = Lb[line * RLS_I + 17 * rrb + n2];
+                    for (int n2 = 0; n2 < 16; ++n2) x[i][n2] = Lb[line * RLS + 17 * rrb + n2];
                     dft_reg<16, true>(x[i]);
                 }
                 if (final) {
@@ -506,7 +515,6 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
 #pragma unroll
                         for (int k2 = 0; k2 < 16; ++k2) __stcs(ph + RB * k2, x[i][k2].x);
                     }
-                    group_sync(g, SGT);
                     continue;
                 }
             }
@@ -548,15 +556,15 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                 }
             }
             // forward pass A on the same registers (cells RB n1 + n2 with n2 = rrb)
-            if (it >= 0) group_sync(g, SGT);  // every inverse pass B has read its cells
+            __syncwarp();  // every inverse pass B (or the slab before) has read its cells
 #pragma unroll
             for (int i = 0; i < NA; ++i) {
                 const int line = lrb + LRBS * i;
                 dft_tw<16, false>(x[i], twa + rrb, RB);
 #pragma unroll
-                for (int k1 = 0; k1 < 16; ++k1) Lb[line * RLS_F + (RB + 1) * k1 + rrb] = x[i][k1];
+                for (int k1 = 0; k1 < 16; ++k1) Lb[line * RLS + (RB + 1) * k1 + rrb] = x[i][k1];
             }
-            group_sync(g, SGT);
+            __syncwarp();
             // forward pass B: cells r16 + 16 k2 of the row spectrum back to memory
             {
                 float2 y[NB][RB];
@@ -564,14 +572,13 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                 for (int i = 0; i < NB; ++i) {
                     const int line = l16 + L16S * i;
 #pragma unroll
-                    for (int n2 = 0; n2 < RB; ++n2) y[i][n2] = Lb[line * RLS_F + (RB + 1) * r16 + n2];
+                    for (int n2 = 0; n2 < RB; ++n2) y[i][n2] = Lb[line * RLS + (RB + 1) * r16 + n2];
                     dft_reg<RB, false>(y[i]);
                     float2* const gp = G + (m0 + line) * N + r16;
 #pragma unroll
                     for (int k2 = 0; k2 < RB; ++k2) __stcg(gp + 16 * k2, y[i][k2]);
                 }
             }
-            group_sync(g, SGT);
         }
         // both groups' rows are in memory before the next column phase (or the next frame)
         if (TEAM) {
