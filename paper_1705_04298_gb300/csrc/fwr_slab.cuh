@@ -40,14 +40,15 @@
 // 8-byte loads and stores: the lanes of a warp take adjacent columns in the
 // column phase, 16 or 32 adjacent cells of a row in the row phase), and
 // shared memory is used only for the exchanges between the passes:
-//   column phase: memory -> pass A -> smem -> pass B -> smem (the partner
-//     bins of the spectral step) -> spectral step and inverse pass A in
-//     registers -> smem -> inverse pass B -> memory;
+//   column phase: memory -> pass A -> smem -> pass B (-> smem, the partner
+//     bins of the spectral step, at 512^2; at 256^2 a thread holds both bins of
+//     a pair) -> spectral step and inverse pass A in registers -> smem ->
+//     inverse pass B -> memory;
 //   row phase: memory -> inverse pass A -> smem -> inverse pass B,
 //     reinsertion, x fill (row sums by warp shuffles) and forward pass A in
 //     registers -> smem -> pass B -> memory.
-// That is six crossings of shared memory per column slab and four per row
-// slab. Column-phase exchanges use lines SN + 1 cells apart, row-phase ones
+// That is four crossings of shared memory per slab, six per column slab at
+// 512^2. Column-phase exchanges use lines SN + 1 cells apart, row-phase ones
 // groups of 16 or RB cells padded by one: all bank-conflict free.
 
 namespace {
@@ -89,9 +90,11 @@ template <int N> struct SlabLayout {
     static constexpr size_t tw = lb + LB_BYTES;             // N cells: w_N^j
     static constexpr size_t a = tw + size_t(N) * 8;         // N cells: a(u)
     static constexpr size_t t = a + size_t(N) * 8;          // N cells: T(u)
-    static constexpr size_t twa = t + size_t(N) * 8;        // 16 x RB cells: w_N^(n2 k1) at [k1][n2]
-    static constexpr size_t twi = twa + size_t(16) * RB * 8;  // RB x 16 cells: w_N^(n2 k1) at [k1][n2]
-    static constexpr size_t pt = twi + size_t(16) * RB * 8;   // 4 N floats
+    // w_N^(n2 k1) at [k1][n2], 16 x RB and RB x 16 cells (256^2: the same table)
+    static constexpr size_t twa = t + size_t(N) * 8;
+    static constexpr size_t twi = N == 256 ? twa : twa + size_t(16) * RB * 8;
+    static constexpr size_t eys = twi + size_t(RB) * 16 * 8;  // 256^2: the groups' fill spectra
+    static constexpr size_t pt = eys + (N == 256 ? size_t(2) * (S2::SC + 1) * 8 : 0);  // 4 N floats
     static constexpr size_t WTS = 2 * size_t(S2::WS) * N > size_t(S1::WS) * N ? 2 * size_t(S2::WS) * N
                                                                                : size_t(S1::WS) * N;
     static constexpr size_t wts = pt + size_t(4) * N * 4;
@@ -202,6 +205,7 @@ struct SlabCtx {
     float2* Tt;
     float2* twa;   // w_N^(n2 k1) at [k1][n2], k1 < 16, n2 < RB (forward pass A)
     float2* twi;   // w_N^(n2 k1) at [k1][n2], k1 < RB, n2 < 16 (inverse pass A)
+    float2* eys;   // 256^2: the groups' y-slope spectra at ky = 0
     float* pt;
     float* wts;    // the groups' weight tables
     const uint8_t* mask;  // shared memory (256^2) or the plan's global copy (512^2)
@@ -221,6 +225,7 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
     c.Tt = reinterpret_cast<float2*>(smem + L::t);
     c.twa = reinterpret_cast<float2*>(smem + L::twa);
     c.twi = reinterpret_cast<float2*>(smem + L::twi);
+    c.eys = reinterpret_cast<float2*>(smem + L::eys);
     c.pt = reinterpret_cast<float*>(smem + L::pt);
     c.wts = reinterpret_cast<float*>(smem + L::wts);
     c.n = n;
@@ -235,8 +240,8 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
     }
     for (int i = tid; i < 4 * N; i += SNT) c.pt[i] = tab.pt[i];
     for (int i = tid; i < 16 * RB; i += SNT) {
-        c.twa[i] = tab.tw[(i % RB) * (i / RB)];  // [k1][n2], k1 < 16
-        c.twi[i] = tab.tw[(i % 16) * (i / 16)];  // [k1][n2], n2 < 16
+        c.twa[i] = tab.tw[(i % RB) * (i / RB)];              // [k1][n2], k1 < 16
+        if (N != 256) c.twi[i] = tab.tw[(i % 16) * (i / 16)];  // [k1][n2], n2 < 16
     }
     if (N == 256) {
         uint8_t* m = smem + L::mask;
@@ -248,6 +253,206 @@ __device__ __forceinline__ void slab_setup(SlabCtx& c, unsigned char* smem, cons
     }
     __syncthreads();
 }
+
+namespace {
+// Algorithm 1 step 2 at the bins k = (ky, kx) and -k, whose values z1, z2 are
+// replaced: Z'(k) = w (a z1 + b conj z2), a = |G|^2/2 + Im P, b = (|Gx|^2 -
+// |Gy|^2)/2 + i Re P, P = Gx conj(Gy) = p(u) conj p(v); at -k Im P and the
+// roles of z1, z2 change. pu: (p(u), |.|^2/2 twice), pv: (p(v), |.|^2 twice).
+__device__ __forceinline__ void lsq_pair(float2& z1, float2& z2, float4 pu, float4 pv, float w) {
+    const float bi = fmadd(pu.x, pv.x, mulrn(pu.y, pv.y)), Py = fmadd(pu.y, pv.x, -mulrn(pu.x, pv.y));
+    const float h2 = mulrn(pu.w, pv.z), S = fmadd(pu.z, pv.w, h2), br = fmadd(pu.z, pv.w, -h2);
+    const float a1 = __fadd_rn(S, Py), a2 = __fsub_rn(S, Py);
+    const float o1x = fmadd(a1, z1.x, fmadd(br, z2.x, mulrn(bi, z2.y)));
+    const float o1y = fmadd(a1, z1.y, fmadd(bi, z2.x, -mulrn(br, z2.y)));
+    const float o2x = fmadd(a2, z2.x, fmadd(br, z1.x, mulrn(bi, z1.y)));
+    const float o2y = fmadd(a2, z2.y, fmadd(bi, z1.x, -mulrn(br, z1.y)));
+    z1 = make_float2(mulrn(w, o1x), mulrn(w, o1y));
+    z2 = make_float2(mulrn(w, o2x), mulrn(w, o2y));
+}
+
+// Eq. 2 with the final filter at k and -k: phi = w (conj(Gx) Sx + conj(Gy) Sy),
+// Hermitian, so the bin at -k takes the conjugate
+__device__ __forceinline__ void final_pair(float2& z1, float2& z2, float2 gx, float2 gy, float w) {
+    const float sxr = __fadd_rn(z1.x, z2.x), sxi = __fsub_rn(z1.y, z2.y);
+    const float syr = __fadd_rn(z1.y, z2.y), syi = __fsub_rn(z2.x, z1.x);
+    const float pr = fmadd(gx.x, sxr, fmadd(gx.y, sxi, fmadd(gy.x, syr, mulrn(gy.y, syi))));
+    const float pi = fmadd(gx.x, sxi, fmadd(-gx.y, sxr, fmadd(gy.x, syi, -mulrn(gy.y, syr))));
+    const float h = mulrn(0.5f, w);
+    z1 = make_float2(mulrn(pr, h), mulrn(pi, h));
+    z2 = make_float2(z1.x, -z1.y);
+}
+
+// y part of Eq. PC at k and -k: Z(k) -= i c, Z(-k) -= i conj(c),
+// c = Sy(0, kx) e^{2 i pi ky / N}; ey = 0 leaves them
+__device__ __forceinline__ void fill_pair(float2& z1, float2& z2, float2 ey, float2 twk) {
+    const float2 c0 = cmulc_rn(twk, ey);
+    z1 = make_float2(__fadd_rn(z1.x, c0.y), __fsub_rn(z1.y, c0.x));
+    z2 = make_float2(__fsub_rn(z2.x, c0.y), __fsub_rn(z2.y, c0.x));
+}
+
+// 256^2 column phase between the exchanges: forward pass B (with the four-step
+// twiddles), the spectral step and inverse pass A of column slab s.
+//
+// A thread holds the bins q + 16 k2 of one column and 16 - q + 16 k2 of its
+// partner column (q = 0: 16 .. 256 there), so bin k's partner -k is in the
+// same thread: no exchange for the spectral step, whose coefficients serve both bins. The
+// columns 0 and N/2 of slab 0 are their own partners: their threads take both
+// tasks in one of the two columns, and those with q = 0 and 8, which hold one
+// task of each column, reorder their registers. 1000 frames of 128 x 128
+// lenslets, k = 10: 6.36 ms with each bin's partner read from shared memory,
+// 5.85 so. (Counting the partner's bins from 16 by its twiddles instead of the
+// register moves takes 5.77 ms but rounds the low frequencies: error 8.6e-7
+// instead of 7.2e-7.) What bounds the kernel: see slab_frame.
+template <int GROUPS>
+__device__ __forceinline__ void column_spectrum(const SlabCtx& c, int s, int g, int tg, bool fill, bool final) {
+    typedef SlabShape<256, GROUPS> Sh;
+    constexpr int N = 256, SC = Sh::SC, WS = Sh::WS, CLS = Sh::CLS, SGT = Sh::SGT;
+    float2* const Lb = c.Lb + g * Sh::LB_CELLS;
+    const float* const wts = c.wts + g * WS * N;
+    float2* const eys = c.eys + g * WS;
+    const float2* const tab = c.twa;
+    const float4* const pt = reinterpret_cast<const float4*>(c.pt);
+    const int cl = tg % SC, q = tg / SC;
+    const bool self = s == 0 && cl == 0, mixed = self && (q & 7) == 0;
+    const int la = self && q > 8 ? SC : cl, lb = self ? ((q & 7) == 0 || q > 8 ? SC : 0) : SC + cl;
+    const int qb = (16 - q) & 15;
+    float2 y[2][16];
+#pragma unroll
+    for (int n2 = 0; n2 < 16; ++n2) y[0][n2] = Lb[la * CLS + 16 * q + n2];
+#pragma unroll
+    for (int n2 = 0; n2 < 16; ++n2) y[1][n2] = Lb[lb * CLS + 16 * qb + n2];
+#pragma unroll
+    for (int n2 = 1; n2 < 16; ++n2) {
+        y[0][n2] = cmul_rn(y[0][n2], tab[16 * n2 + q]);
+        y[1][n2] = cmul_rn(y[1][n2], tab[16 * n2 + qb]);
+    }
+    dft_reg<16, false>(y[0]);
+    dft_reg<16, false>(y[1]);
+    if (q == 0) {
+        // bins 16 .. 256 of the partner column instead of 0 .. 240
+        const float2 v = y[1][0];
+#pragma unroll
+        for (int k = 0; k < 15; ++k) y[1][k] = y[1][k + 1];
+        y[1][15] = v;
+        // Sy(0, kx) = (Z(0, kx) - conj Z(0, -kx)) / (2i)
+        const float2 e0 = y[0][0], e1 = y[1][15];
+        const float on = fill ? 1.f : 0.f;
+        if (self) {
+            eys[0] = make_float2(on * e0.y, 0.f);
+            eys[SC] = make_float2(on * e1.y, 0.f);
+        } else {
+            eys[cl] = make_float2(on * 0.5f * (e0.y + e1.y), on * 0.5f * (e1.x - e0.x));
+        }
+    }
+    cp_wait_all();
+    group_sync(g, SGT);
+    // the frequency of bin y[0][k2]: kx(k2 / 8), ky = q + 16 k2; its partner y[1][15 - k2]
+    const int col0 = self && q > 8 ? SC : cl, col1 = mixed ? SC : col0;
+    const int kx0 = col0 == SC ? N / 2 : SC * s + col0, kx1 = col1 == SC ? N / 2 : SC * s + col1;
+    float2 m0 = make_float2(0.f, 0.f), m1 = m0;
+    if (mixed) {
+        if (q == 8) {
+#pragma unroll
+            for (int k = 8; k < 16; ++k) {
+                const float2 v = y[0][k];
+                y[0][k] = y[1][k];
+                y[1][k] = v;
+            }
+        } else {
+            // bins (128, 0) and (0, 128) have no slot in the pairing
+            m0 = y[0][8];
+            m1 = y[1][15];
+            float2 v[7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) v[k] = y[0][9 + k];
+#pragma unroll
+            for (int k = 15; k >= 8; --k) y[0][k] = y[1][k - 1];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) y[1][8 + k] = v[k];
+            y[1][15] = y[0][0];
+            float2 d0 = m0, d1 = m1;
+            fill_pair(m0, d0, eys[0], c.tw[N / 2]);
+            fill_pair(m1, d1, eys[SC], c.tw[0]);
+            d0 = m0;
+            d1 = m1;
+            if (!final) {
+                float4 p0 = pt[0], pm = pt[N / 2];
+                const float4 r0 = p0, rm = pm;
+                p0.z *= 0.5f, p0.w *= 0.5f, pm.z *= 0.5f, pm.w *= 0.5f;
+                lsq_pair(m0, d0, p0, rm, wts[(N / 2) * WS]);
+                lsq_pair(m1, d1, pm, r0, wts[SC]);
+            } else {
+                final_pair(m0, d0, cmul_rn(c.A[0], c.Tt[N / 2]), cmul_rn(c.Tt[0], c.A[N / 2]), wts[(N / 2) * WS]);
+                final_pair(m1, d1, cmul_rn(c.A[N / 2], c.Tt[0]), cmul_rn(c.Tt[N / 2], c.A[0]), wts[SC]);
+            }
+        }
+    }
+    if (!final) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int kx = h ? kx1 : kx0, col = h ? col1 : col0;
+            const float2 ey = eys[col];
+            float4 pu = pt[kx];
+            pu.z *= 0.5f;
+            pu.w *= 0.5f;
+#pragma unroll
+            for (int k2 = 8 * h; k2 < 8 * h + 8; ++k2) {
+                const int ky = q + 16 * k2;
+                fill_pair(y[0][k2], y[1][15 - k2], ey, c.tw[ky]);
+                lsq_pair(y[0][k2], y[1][15 - k2], pu, pt[ky], wts[ky * WS + col]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int kx = h ? kx1 : kx0, col = h ? col1 : col0;
+            const float2 ey = eys[col], Akx = c.A[kx], Tkx = c.Tt[kx];
+#pragma unroll
+            for (int k2 = 8 * h; k2 < 8 * h + 8; ++k2) {
+                const int ky = q + 16 * k2;
+                fill_pair(y[0][k2], y[1][15 - k2], ey, c.tw[ky]);
+                final_pair(y[0][k2], y[1][15 - k2], cmul_rn(Akx, c.Tt[ky]), cmul_rn(Tkx, c.A[ky]), wts[ky * WS + col]);
+            }
+        }
+    }
+    if (mixed) {
+        if (q == 8) {
+#pragma unroll
+            for (int k = 8; k < 16; ++k) {
+                const float2 v = y[0][k];
+                y[0][k] = y[1][k];
+                y[1][k] = v;
+            }
+        } else {
+            float2 v[7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) v[k] = y[1][8 + k];
+#pragma unroll
+            for (int k = 8; k < 15; ++k) y[1][k] = y[0][k + 1];
+            y[1][15] = m1;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) y[0][9 + k] = v[k];
+            y[0][8] = m0;
+        }
+    }
+    if (q == 0) {
+        const float2 v = y[1][15];
+#pragma unroll
+        for (int k = 15; k > 0; --k) y[1][k] = y[1][k - 1];
+        y[1][0] = v;
+    }
+    // inverse pass A: the bins 16 n1 + q (and 16 n1 + 16 - q of the partner)
+    dft_reg<16, true>(y[0]);
+    dft_reg<16, true>(y[1]);
+#pragma unroll
+    for (int k1 = 0; k1 < 16; ++k1) {
+        Lb[la * CLS + 16 * k1 + q] = k1 ? cmulc_rn(tab[16 * k1 + q], y[0][k1]) : y[0][k1];
+        Lb[lb * CLS + 16 * k1 + qb] = k1 ? cmulc_rn(tab[16 * k1 + qb], y[1][k1]) : y[1][k1];
+    }
+}
+
+}  // namespace
 
 // One frame through the whole path with the grid in G (this CTA's N^2
 // scratch area). TEAM: the bar.team CTAs share the frame and G; CTA `rank`
@@ -285,6 +490,7 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
     const float2* const Tt = c.Tt;
     const float* const pt = c.pt;
     float* const wts = c.wts + g * WS * N;
+    constexpr bool PAIRED = N == 256;
     const uint8_t* const mask = c.mask;
     const int n = c.n, off = c.off, nn = c.nn, mode = c.mode;
     bool finite = true;
@@ -330,7 +536,8 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
 #pragma unroll
                     for (int i = 0; i < NA; ++i) {
                         const int n2 = cq + CQS * i;
-                        dft_tw<16, false>(x[i], twa + n2, RB);
+                        if (PAIRED) dft_reg<16, false>(x[i]);  // twiddles: pass B
+                        else dft_tw<16, false>(x[i], twa + n2, RB);
                         // the slab before: every inverse pass B has read its cells
                         if (i == 0) group_sync(g, SGT);
 #pragma unroll
@@ -338,84 +545,88 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                     }
                 }
                 group_sync(g, SGT);
-                // pass B: bins ky = k1 + 16 k2 of the column
-                float2 y[NB][RB];
+                if constexpr (PAIRED) {
+                    column_spectrum<GROUPS>(c, s, g, tg, fill, final);
+                } else {
+                    // pass B: bins ky = k1 + 16 k2 of the column
+                    float2 y[NB][RB];
 #pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int k1 = cq + CQS * i;
+                    for (int i = 0; i < NB; ++i) {
+                        const int k1 = cq + CQS * i;
 #pragma unroll
-                    for (int n2 = 0; n2 < RB; ++n2) y[i][n2] = Lb[cl * CLS + RB * k1 + n2];
-                    dft_reg<RB, false>(y[i]);
-                }
-                group_sync(g, SGT);
-                // the spectrum in natural order, for the partner bins
-#pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int k1 = cq + CQS * i;
-#pragma unroll
-                    for (int k2 = 0; k2 < RB; ++k2) Lb[cl * CLS + k1 + 16 * k2] = y[i][k2];
-                }
-                cp_wait_all();
-                group_sync(g, SGT);
-                // spectral step on the task's own bins (ky, kx), partner (-ky, -kx) from
-                // shared memory; then the inverse pass A on the same registers
-                float2 ey = make_float2(0.f, 0.f);
-                if (fill) {
-                    // Sy(0, kx) = (Z(0, kx) - conj Z(0, -kx)) / (2i), uncorrected values
-                    const float2 e0 = Lb[cl * CLS], e1 = Lb[pl * CLS];
-                    ey = make_float2(0.5f * (e0.y + e1.y), 0.5f * (e1.x - e0.x));
-                }
-                const float4 pu = *reinterpret_cast<const float4*>(pt + 4 * kx);
-                const float2 Akx = A[kx], Tkx = Tt[kx];
-                // weight column of this line and whether its rows are mirrored
-                const bool first = cl < SC || (s == 0 && cl == SC);
-                const int wcol = (s == 0 && cl == SC) ? SC : (cl % SC);
-#pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int k1 = cq + CQS * i;
-#pragma unroll
-                    for (int k2 = 0; k2 < RB; ++k2) {
-                        const int ky = k1 + 16 * k2, kyn = (N - ky) & (N - 1);
-                        float2 z1 = y[i][k2], z2 = Lb[pl * CLS + kyn];
-                        if (fill) {
-                            // y part of Eq. PC: Z(k) -= i c, Z(-k) -= i conj(c),
-                            // c = Sy(0, kx) e^{2 i pi ky / N}
-                            const float2 c0 = cmul(ey, conjf2(tw[ky]));
-                            z1 = make_float2(z1.x + c0.y, z1.y - c0.x);
-                            z2 = make_float2(z2.x - c0.y, z2.y - c0.x);
-                        }
-                        const float w = wts[(first ? ky : kyn) * WS + wcol];
-                        const float4 pv = *reinterpret_cast<const float4*>(pt + 4 * ky);
-                        if (!final) {
-                            // Algorithm 1 step 2: Z'(k) = w (a z1 + b conj z2) with, at the
-                            // bin's own frequency, a = |G|^2/2 + Im P, b = (|Gx|^2 - |Gy|^2)/2
-                            // + i Re P, P = Gx conj(Gy) = p(u) conj p(v)
-                            const float Px = pu.x * pv.x + pu.y * pv.y, Py = pu.y * pv.x - pu.x * pv.y;
-                            const float h1 = 0.5f * pu.z * pv.w, h2 = 0.5f * pu.w * pv.z;
-                            const float a = h1 + h2 + Py, br = h1 - h2, bi = Px;
-                            const float ox = a * z1.x + br * z2.x + bi * z2.y;
-                            const float oy = a * z1.y + bi * z2.x - br * z2.y;
-                            y[i][k2] = make_float2(w * ox, w * oy);
-                        } else {
-                            // Eq. 2 with the final filter: phi = w (conj(Gx) Sx + conj(Gy) Sy)
-                            const float2 z2c = conjf2(z2);
-                            const float2 sx = make_float2(0.5f * (z1.x + z2c.x), 0.5f * (z1.y + z2c.y));
-                            const float2 sy = make_float2(0.5f * (z1.y - z2c.y), 0.5f * (z2c.x - z1.x));
-                            const float2 gx = cmul(Akx, Tt[ky]);
-                            const float2 gy = cmul(Tkx, A[ky]);
-                            const float2 ph = cadd(cmulc(gx, sx), cmulc(gy, sy));
-                            y[i][k2] = make_float2(ph.x * w, ph.y * w);
-                        }
+                        for (int n2 = 0; n2 < RB; ++n2) y[i][n2] = Lb[cl * CLS + RB * k1 + n2];
+                        dft_reg<RB, false>(y[i]);
                     }
-                    // inverse pass A: the bins ky = 16 n1 + n2 with n2 = k1
-                    dft_tw<RB, true>(y[i], twi + k1, 16);
-                }
-                group_sync(g, SGT);
+                    group_sync(g, SGT);
+                    // the spectrum in natural order, for the partner bins
 #pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int n2 = cq + CQS * i;
+                    for (int i = 0; i < NB; ++i) {
+                        const int k1 = cq + CQS * i;
 #pragma unroll
-                    for (int k1 = 0; k1 < RB; ++k1) Lb[cl * CLS + 16 * k1 + n2] = y[i][k1];
+                        for (int k2 = 0; k2 < RB; ++k2) Lb[cl * CLS + k1 + 16 * k2] = y[i][k2];
+                    }
+                    cp_wait_all();
+                    group_sync(g, SGT);
+                    // spectral step on the task's own bins (ky, kx), partner (-ky, -kx) from
+                    // shared memory; then the inverse pass A on the same registers
+                    float2 ey = make_float2(0.f, 0.f);
+                    if (fill) {
+                        // Sy(0, kx) = (Z(0, kx) - conj Z(0, -kx)) / (2i), uncorrected values
+                        const float2 e0 = Lb[cl * CLS], e1 = Lb[pl * CLS];
+                        ey = make_float2(0.5f * (e0.y + e1.y), 0.5f * (e1.x - e0.x));
+                    }
+                    const float4 pu = *reinterpret_cast<const float4*>(pt + 4 * kx);
+                    const float2 Akx = A[kx], Tkx = Tt[kx];
+                    // weight column of this line and whether its rows are mirrored
+                    const bool first = cl < SC || (s == 0 && cl == SC);
+                    const int wcol = (s == 0 && cl == SC) ? SC : (cl % SC);
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const int k1 = cq + CQS * i;
+#pragma unroll
+                        for (int k2 = 0; k2 < RB; ++k2) {
+                            const int ky = k1 + 16 * k2, kyn = (N - ky) & (N - 1);
+                            float2 z1 = y[i][k2], z2 = Lb[pl * CLS + kyn];
+                            if (fill) {
+                                // y part of Eq. PC: Z(k) -= i c, Z(-k) -= i conj(c),
+                                // c = Sy(0, kx) e^{2 i pi ky / N}
+                                const float2 c0 = cmul(ey, conjf2(tw[ky]));
+                                z1 = make_float2(z1.x + c0.y, z1.y - c0.x);
+                                z2 = make_float2(z2.x - c0.y, z2.y - c0.x);
+                            }
+                            const float w = wts[(first ? ky : kyn) * WS + wcol];
+                            const float4 pv = *reinterpret_cast<const float4*>(pt + 4 * ky);
+                            if (!final) {
+                                // Algorithm 1 step 2: Z'(k) = w (a z1 + b conj z2) with, at the
+                                // bin's own frequency, a = |G|^2/2 + Im P, b = (|Gx|^2 - |Gy|^2)/2
+                                // + i Re P, P = Gx conj(Gy) = p(u) conj p(v)
+                                const float Px = pu.x * pv.x + pu.y * pv.y, Py = pu.y * pv.x - pu.x * pv.y;
+                                const float h1 = 0.5f * pu.z * pv.w, h2 = 0.5f * pu.w * pv.z;
+                                const float a = h1 + h2 + Py, br = h1 - h2, bi = Px;
+                                const float ox = a * z1.x + br * z2.x + bi * z2.y;
+                                const float oy = a * z1.y + bi * z2.x - br * z2.y;
+                                y[i][k2] = make_float2(w * ox, w * oy);
+                            } else {
+                                // Eq. 2 with the final filter: phi = w (conj(Gx) Sx + conj(Gy) Sy)
+                                const float2 z2c = conjf2(z2);
+                                const float2 sx = make_float2(0.5f * (z1.x + z2c.x), 0.5f * (z1.y + z2c.y));
+                                const float2 sy = make_float2(0.5f * (z1.y - z2c.y), 0.5f * (z2c.x - z1.x));
+                                const float2 gx = cmul(Akx, Tt[ky]);
+                                const float2 gy = cmul(Tkx, A[ky]);
+                                const float2 ph = cadd(cmulc(gx, sx), cmulc(gy, sy));
+                                y[i][k2] = make_float2(ph.x * w, ph.y * w);
+                            }
+                        }
+                        // inverse pass A: the bins ky = 16 n1 + n2 with n2 = k1
+                        dft_tw<RB, true>(y[i], twi + k1, 16);
+                    }
+                    group_sync(g, SGT);
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const int n2 = cq + CQS * i;
+#pragma unroll
+                        for (int k1 = 0; k1 < RB; ++k1) Lb[cl * CLS + 16 * k1 + n2] = y[i][k1];
+                    }
                 }
                 group_sync(g, SGT);
                 // inverse pass B, rows k1 + RB k2 of the column back to memory

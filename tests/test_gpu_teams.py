@@ -2,9 +2,12 @@
 frame gives bitwise the phase of the same kernel with one CTA per frame (an
 explicit persistent-grid size, FWR_OPT_CTAS, keeps that one)."""
 
+import numpy as np
 import pytest
 
+import oracle
 from paper_1705_04298_gb300 import synth
+from parity_check import FP32_RMS, within
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -77,3 +80,19 @@ def test_teams_report_nonfinite_slopes(fwr):
     plan.reconstruct(s, 1)
     assert plan.status() == "FWR_ERR_NONFINITE"
     assert plan.status() == "FWR_OK"
+
+
+# a white warm start reaches every bin pair of the 256^2 spectral step: the
+# self-paired columns 0 and 128, their self-paired bins, every fill mode
+@pytest.mark.parametrize("n,k,periodic", [(128, 1, 0), (101, 2, 1), (160, 1, 2), (77, 0, 0)])
+@pytest.mark.parametrize("shape", [0, 1])
+def test_256_every_bin(fwr, n, k, periodic, shape):
+    s, mask = frames(n, 1, 60 + n)
+    plan = fwr.Plan(mask, 1.0, fwr.WIENER, 0.01, 0.6, 100.0, periodic, grid=256)
+    plan.set_shape(shape)
+    ext = np.random.default_rng(n).standard_normal((1, 2, 256, 256)).astype(np.float32)
+    ph = plan.reconstruct(s, k, ext_init=torch.tensor(ext, device="cuda"))
+    assert plan.status() == "FWR_OK"
+    ref, _ = oracle.reconstruct(s[0].cpu().double().numpy(), mask, 1.0, k, oracle.FILTER_WIENER, 0.01, 0.6, 100.0, periodic,
+                                ext_init=ext[0].astype(np.float64), N=256)
+    assert within(ph[0].cpu().numpy(), ref, FP32_RMS, where="n=%d" % n)
