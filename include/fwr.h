@@ -435,8 +435,11 @@ void fwr_ragged_release(void);
  *                    tensor cores (implicit GEMM, BF16 in, FP32 accumulate);
  *                    FWR_NET_CONV_SIMT keeps every convolution on the CUDA
  *                    cores. Both sum in FP32 and round the stored activation to
- *                    BF16; they differ only in summation order. Unknown option
- *                    or value: FWR_ERR_ARG.
+ *                    BF16; they differ only in summation order. The same holds
+ *                    for the backward pass, whose FP32 gradients enter the
+ *                    tensor cores as three exact BF16 parts (layers with input
+ *                    and output channels multiples of 16). Unknown option or
+ *                    value: FWR_ERR_ARG.
  * fwr_net_tc_layers  how many layers are eligible for the tensor-core forward
  *                    (-1 for NULL).
  */

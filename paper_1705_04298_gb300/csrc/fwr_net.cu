@@ -494,7 +494,7 @@ cudaError_t forward(fwr_net* n, int Bn, cudaStream_t s) {
 cudaError_t conv_bwd(fwr_net* n, int li, const float* dZ, const bf16* A, const bf16* B, int Bn, const bf16* act,
                      float* din, float* lo, const bf16* lo_act, cudaStream_t s) {
     const Layer& L = n->layers[li];
-    const ConvBwd c{L.ca, L.cb, L.cout, L.H, L.upA, A, B};
+    const ConvBwd c{L.ca, L.cb, L.cout, L.H, L.upA, A, B, n->conv == FWR_NET_CONV_SIMT};
     cudaError_t e = conv_wgrad(c, dZ, Bn, n->gws, n->G + L.woff, n->sms, s);
     if (e == cudaSuccess && din) e = conv_dgrad(c, dZ, n->Wb + L.woff, Bn, act, din, lo, lo_act, n->sms, s);
     return e;
@@ -665,7 +665,7 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
     for (const Layer& L : n->layers) {
         if (L.k != 3) continue;
         gws = std::max(gws, wgrad_ws_floats(L.ca + L.cb, L.cout, L.H, n->sms));
-        if (e == cudaSuccess && !netgrad_prepare(L.ca + L.cb, L.cout, L.H)) e = cudaErrorInvalidValue;
+        if (e == cudaSuccess && !netgrad_prepare(L.ca, L.cb, L.cout, L.H)) e = cudaErrorInvalidValue;
     }
     if (e == cudaSuccess) e = cudaMalloc(&n->gws, gws * sizeof(float));
     falloc(&n->dpool, B * 16 * 16 * w1 + B * 8 * 8 * w2 + B * 4 * 4 * w3);

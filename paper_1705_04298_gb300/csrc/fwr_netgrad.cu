@@ -1,14 +1,16 @@
 // Backward pass of the warm-start network's convolutions (sm_103a).
 //
 // Weight gradients and input gradients are contractions with one FP32 operand
-// (the activations' gradients stay FP32; weights and activations are BF16), so
-// they run on the FP32 pipe, with the packed two-lane FMA (fma.rn.f32x2, half
-// the issue slots of scalar FMA at the same lane rate). What bounds them is
-// that pipe: 19 GFLOP each for 256 images at width 16, 0.25 ms at 78 TFLOP/s.
-// Each thread keeps a register tile whose operands come from shared memory in
-// 16-byte loads, few loads per FMA. Measured on 256 images at width 16, the
-// whole gradient call: 90.6 ms with scalar kernels (one block per output
-// channel and tap, operands from global memory), 2.5 ms with these.
+// (the activations' gradients stay FP32; weights and activations are BF16).
+// Layers whose channel counts are multiples of 16 take the tensor-core kernels
+// of fwr_netgradtc.cu; the others (at the shipped width 16 only the first
+// layer, three input channels) run here on the FP32 pipe, with the packed
+// two-lane FMA (fma.rn.f32x2, half the issue slots of scalar FMA at the same
+// lane rate), which bounds them. Each thread keeps a register tile whose
+// operands come from shared memory in 16-byte loads, few loads per FMA.
+// Measured on 256 images at width 16, the whole gradient call: 90.6 ms with
+// scalar kernels (one block per output channel and tap, operands from global
+// memory), 2.5 ms with these, 1.06 ms with the tensor cores'.
 
 #include <stdint.h>
 
@@ -293,15 +295,18 @@ k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int
 __global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ ws, int chunks, int n, float* g, float* last) {
     __shared__ float part[8][33];
     const int c = threadIdx.x & 31, q = threadIdx.x >> 5, i = blockIdx.x * 32 + c;
-    float v = 0.f;
+    float u[4] = {0.f, 0.f, 0.f, 0.f};
     if (i < n) {
-#pragma unroll 4
-        for (int k = q; k < chunks; k += 8) v += ws[size_t(k) * n + i];
+        for (int k = q; k < chunks; k += 32)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (k + 8 * j < chunks) u[j] += ws[size_t(k + 8 * j) * n + i];
     }
-    part[q][c] = v;
+    part[q][c] = (u[0] + u[1]) + (u[2] + u[3]);
     __syncthreads();
     if (q == 0 && i < n) {
-        for (int k = 1; k < 8; ++k) v += part[k][c];
+        const float v = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) +
+                        ((part[4][c] + part[5][c]) + (part[6][c] + part[7][c]));
         if (last && i == n - 1) *last = v;
         else g[i] = v;
     }
@@ -597,23 +602,31 @@ int out_ctas(int sms) { return 4 * sms; }
 
 size_t wgrad_ws_floats(int cin, int cout, int H, int sms) {
     const WgradShape w = wgrad_shape(cin, cout, H);
-    return size_t(std::max(1, 2 * sms / w.ny)) * (size_t(cout) * 9 * cin + cout);
+    const size_t n = size_t(std::max(1, 2 * sms / w.ny)) * (size_t(cout) * 9 * cin + cout);
+    return cin % 16 == 0 && cout % 16 == 0 ? std::max(n, wgrad_tc_ws_floats(cin, cout, H, sms)) : n;
 }
 
 cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, float* g, int sms, cudaStream_t s) {
-    const int cin = L.ca + L.cb, rows = Bn * L.H;
+    const int cin = L.ca + L.cb, rows = Bn * L.H, n = L.cout * 9 * cin + L.cout;
+    if (wgrad_tc_fits(L, dZ)) {
+        int chunks = 0;
+        const cudaError_t e = wgrad_tc(L, dZ, Bn, ws, &chunks, sms, s);
+        if (e != cudaSuccess) return e;
+        k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, chunks, n, g, nullptr);
+        return cudaGetLastError();
+    }
     const WgradShape w = wgrad_shape(cin, L.cout, L.H);
     const int rc = wgrad_rows(w, rows, sms), chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad3<32> : L.H == 16 ? k_wgrad3<16> : L.H == 8 ? k_wgrad3<8> : k_wgrad3<4>;
     kern<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                        ws);
-    const int n = L.cout * 9 * cin + L.cout;
     k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, chunks, n, g, nullptr);
     return cudaGetLastError();
 }
 
 cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
                        float* lo, const bf16* lo_act, int sms, cudaStream_t s) {
+    if (dgrad_tc_fits(L, dZ, Wt)) return dgrad_tc(L, dZ, Wt, Bn, act, dIn, lo, lo_act, sms, s);
     const int pairs = Bn * (L.H / 2);
     const DgradShape d = dgrad_shape(L.ca + L.cb, L.H, pairs, sms);
     auto kern = L.H == 32 ? k_dgrad3<32> : L.H == 16 ? k_dgrad3<16> : L.H == 8 ? k_dgrad3<8> : k_dgrad3<4>;
@@ -635,9 +648,10 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
     return cudaGetLastError();
 }
 
-bool netgrad_prepare(int cin, int cout, int H) {
-    const int lim = 227 * 1024;
+bool netgrad_prepare(int ca, int cb, int cout, int H) {
+    const int lim = 227 * 1024, cin = ca + cb;
     if (H != 32 && H != 16 && H != 8 && H != 4) return false;
+    if (grad_tc_shape(ca, cb, cout) && !grad_tc_prepare(cin, cout, H)) return false;
     if (std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H, 1ll << 40, 1).smem) > size_t(lim)) return false;
     cudaError_t e = cudaSuccess;
     for (auto k : {k_wgrad3<32>, k_wgrad3<16>, k_wgrad3<8>, k_wgrad3<4>})

@@ -17,6 +17,7 @@ struct ConvBwd {
     int ca, cb, cout, H;
     bool upA;
     const bf16 *A, *B;
+    bool simt;  // FP32 pipe only
 };
 
 // dW, db of a 3 x 3 layer into g (flat: W[cout][3][3][cin], then the biases),
@@ -32,6 +33,18 @@ size_t wgrad_ws_floats(int cin, int cout, int H, int sms);
 cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
                        float* lo, const bf16* lo_act, int sms, cudaStream_t s);
 
+// Tensor-core forms of the two (fwr_netgradtc.cu), which conv_wgrad and
+// conv_dgrad take for layers whose channel counts are multiples of 16;
+// wgrad_tc leaves the sums of *chunks parts in ws.
+bool grad_tc_shape(int ca, int cb, int cout);
+bool grad_tc_prepare(int cin, int cout, int H);
+size_t wgrad_tc_ws_floats(int cin, int cout, int H, int sms);
+bool wgrad_tc_fits(const ConvBwd& L, const float* dZ);
+cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* chunks, int sms, cudaStream_t s);
+bool dgrad_tc_fits(const ConvBwd& L, const float* dZ, const bf16* Wt);
+cudaError_t dgrad_tc(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
+                     float* lo, const bf16* lo_act, int sms, cudaStream_t s);
+
 // Masked mean squared error of pred against T and the backward of the 1 x 1
 // output layer (C input channels a, two outputs): dIn [npix][C] (zeroed where
 // a is not positive), g = W[2][C], b[2] gradients, *loss.
@@ -41,7 +54,7 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
 size_t out_ws_floats(int C, int sms);
 
 // shared-memory limits of the kernels above for a layer; false if it cannot run
-bool netgrad_prepare(int cin, int cout, int H);
+bool netgrad_prepare(int ca, int cb, int cout, int H);
 
 }  // namespace net
 }  // namespace fwr

@@ -158,6 +158,41 @@ def test_gradients_at_other_widths(fwr, w, F):
     assert rel <= 5e-2, rel
 
 
+@pytest.mark.parametrize("w,F", [(16, 1), (16, 3), (16, 37), (16, 260), (8, 9), (32, 5)])
+def test_gradients_tensor_cores_match_cuda_cores(fwr, w, F):
+    """The tensor-core backward kernels against the CUDA-core ones, layer by
+    layer, for batches that leave remainders in both kernels' pixel tiles and
+    for widths with layers of either kind. The inputs are multiples of 1/4 and
+    every output has four weights of +-1, so all forward sums are exact in any
+    order and both runs have the same activations and loss; the gradients then
+    differ by FP32 summation only, at most about 3e-7 of a layer's norm per
+    kernel, two kernels a layer, 14 layers deep: 1e-5."""
+    rng = np.random.default_rng(w + F)
+    parts = []
+    for name, ci, co, k in unet.layer_specs(w):
+        m = np.zeros((co, k * k * ci), np.float32)
+        for row in m:
+            row[rng.choice(k * k * ci, 4, replace=False)] = rng.choice((-1.0, 1.0), 4)
+        parts += [m.ravel(), np.zeros(co, np.float32)]
+    n = 40
+    mask = synth.pupil_mask(n)
+    plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=128)
+    net = fwr.Net(w, F, np.concatenate(parts))
+    s = torch.tensor(rng.integers(-8, 9, (F, 2, n, n)) * (0.25 * mask), dtype=torch.float32, device="cuda")
+    e = torch.tensor(rng.standard_normal((F, 2, 128, 128)), dtype=torch.float32, device="cuda")
+    loss, g = net.gradients(plan, s, e)
+    net.set_conv(fwr.NET_CONV_SIMT)
+    loss_s, g_s = net.gradients(plan, s, e)
+    assert loss == loss_s
+    pos = 0
+    for name, ci, co, k in unet.layer_specs(w):
+        m = co * k * k * ci + co
+        a, b = g[pos:pos + m].astype(np.float64), g_s[pos:pos + m].astype(np.float64)
+        pos += m
+        assert np.linalg.norm(b) > 0, name
+        assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b), (name, np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
 @pytest.mark.parametrize("n,F", [(40, 1), (37, 5), (64, 307)])
 def test_one_kernel_forward_matches_layers(fwr, n, F):
     """Width 16: the one-kernel forward (more images than it has CTAs in the
