@@ -2,15 +2,15 @@
 //
 // Weight gradients and input gradients are contractions with one FP32 operand
 // (the activations' gradients stay FP32; weights and activations are BF16).
-// Layers whose channel counts are multiples of 16 take the tensor-core kernels
-// of fwr_netgradtc.cu; the others (at the shipped width 16 only the first
-// layer, three input channels) run here on the FP32 pipe, with the packed
-// two-lane FMA (fma.rn.f32x2, half the issue slots of scalar FMA at the same
-// lane rate), which bounds them. Each thread keeps a register tile whose
+// Layers whose channel counts are multiples of 16 (and the first layer, three
+// input channels) take the tensor-core kernels of fwr_netgradtc.cu; those of
+// other widths run here on the FP32 pipe, with the packed two-lane FMA
+// (fma.rn.f32x2, half the issue slots of scalar FMA at the same lane rate),
+// which bounds them. Each thread keeps a register tile whose
 // operands come from shared memory in 16-byte loads, few loads per FMA.
 // Measured on 256 images at width 16, the whole gradient call: 90.6 ms with
 // scalar kernels (one block per output channel and tap, operands from global
-// memory), 2.5 ms with these, 1.06 ms with the tensor cores'.
+// memory), 2.5 ms with these, 1.01 ms with the tensor cores'.
 
 #include <stdint.h>
 
@@ -291,25 +291,39 @@ k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int
 }
 
 // g[i] = sum over chunks of ws[chunk][i]; the last of `n` sums goes to *last
-// when given. 32 sums x 8 chunk lanes per block.
-__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ ws, int chunks, int n, float* g, float* last) {
-    __shared__ float part[8][33];
+// when given. 32 sums x LANES chunk lanes per block, four of a lane's loads in
+// flight together: 32 lanes where there are few sums (2320 sums of 304 chunks:
+// 5 us, 8 with 8 lanes), 8 where the blocks fill the chip (36928 sums of 147:
+// 7.5 us, 12 with 32).
+template <int LANES>
+__global__ void __launch_bounds__(32 * LANES)
+k_reduce(const float* __restrict__ ws, int chunks, int n, float* g, float* last) {
+    __shared__ float part[LANES][33];
     const int c = threadIdx.x & 31, q = threadIdx.x >> 5, i = blockIdx.x * 32 + c;
     float u[4] = {0.f, 0.f, 0.f, 0.f};
     if (i < n) {
-        for (int k = q; k < chunks; k += 32)
+        for (int k = q; k < chunks; k += 4 * LANES)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (k + 8 * j < chunks) u[j] += ws[size_t(k + 8 * j) * n + i];
+                if (k + LANES * j < chunks) u[j] += ws[size_t(k + LANES * j) * n + i];
     }
     part[q][c] = (u[0] + u[1]) + (u[2] + u[3]);
     __syncthreads();
-    if (q == 0 && i < n) {
-        const float v = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) +
-                        ((part[4][c] + part[5][c]) + (part[6][c] + part[7][c]));
-        if (last && i == n - 1) *last = v;
-        else g[i] = v;
+#pragma unroll
+    for (int h = LANES / 2; h > 0; h /= 2) {
+        if (q < h) part[q][c] += part[q + h][c];
+        __syncthreads();
     }
+    if (q == 0 && i < n) {
+        if (last && i == n - 1) *last = part[0][c];
+        else g[i] = part[0][c];
+    }
+}
+cudaError_t reduce_chunks(const float* ws, int chunks, int n, float* g, float* last, int sms, cudaStream_t s) {
+    const int blocks = (n + 31) / 32;
+    if (blocks < 2 * sms) k_reduce<32><<<blocks, 1024, 0, s>>>(ws, chunks, n, g, last);
+    else k_reduce<8><<<blocks, 256, 0, s>>>(ws, chunks, n, g, last);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- input gradient
@@ -603,7 +617,7 @@ int out_ctas(int sms) { return 4 * sms; }
 size_t wgrad_ws_floats(int cin, int cout, int H, int sms) {
     const WgradShape w = wgrad_shape(cin, cout, H);
     const size_t n = size_t(std::max(1, 2 * sms / w.ny)) * (size_t(cout) * 9 * cin + cout);
-    return cin % 16 == 0 && cout % 16 == 0 ? std::max(n, wgrad_tc_ws_floats(cin, cout, H, sms)) : n;
+    return (cin % 16 == 0 || cin < 16) && cout % 16 == 0 ? std::max(n, wgrad_tc_ws_floats(cin, cout, H, sms)) : n;
 }
 
 cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, float* g, int sms, cudaStream_t s) {
@@ -611,17 +625,14 @@ cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, flo
     if (wgrad_tc_fits(L, dZ)) {
         int chunks = 0;
         const cudaError_t e = wgrad_tc(L, dZ, Bn, ws, &chunks, sms, s);
-        if (e != cudaSuccess) return e;
-        k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, chunks, n, g, nullptr);
-        return cudaGetLastError();
+        return e == cudaSuccess ? reduce_chunks(ws, chunks, n, g, nullptr, sms, s) : e;
     }
     const WgradShape w = wgrad_shape(cin, L.cout, L.H);
     const int rc = wgrad_rows(w, rows, sms), chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad3<32> : L.H == 16 ? k_wgrad3<16> : L.H == 8 ? k_wgrad3<8> : k_wgrad3<4>;
     kern<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                        ws);
-    k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, chunks, n, g, nullptr);
-    return cudaGetLastError();
+    return reduce_chunks(ws, chunks, n, g, nullptr, sms, s);
 }
 
 cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
@@ -644,14 +655,13 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
     k_out_bwd<<<used, 256, 0, s>>>(reinterpret_cast<const float2*>(pred), reinterpret_cast<const float2*>(T), LM, cnt,
                                    npix, per, C, a, Wt, dIn, ws);
     const int n = 2 * C + 3;
-    k_reduce<<<(n + 31) / 32, 256, 0, s>>>(ws, used, n, g, loss);
-    return cudaGetLastError();
+    return reduce_chunks(ws, used, n, g, loss, sms, s);
 }
 
 bool netgrad_prepare(int ca, int cb, int cout, int H) {
     const int lim = 227 * 1024, cin = ca + cb;
     if (H != 32 && H != 16 && H != 8 && H != 4) return false;
-    if (grad_tc_shape(ca, cb, cout) && !grad_tc_prepare(cin, cout, H)) return false;
+    if ((wgrad_tc_shape(ca, cb, cout) || dgrad_tc_shape(ca, cb, cout)) && !grad_tc_prepare(cin, cout, H)) return false;
     if (std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H, 1ll << 40, 1).smem) > size_t(lim)) return false;
     cudaError_t e = cudaSuccess;
     for (auto k : {k_wgrad3<32>, k_wgrad3<16>, k_wgrad3<8>, k_wgrad3<4>})

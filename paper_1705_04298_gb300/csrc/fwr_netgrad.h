@@ -34,9 +34,10 @@ cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn
                        float* lo, const bf16* lo_act, int sms, cudaStream_t s);
 
 // Tensor-core forms of the two (fwr_netgradtc.cu), which conv_wgrad and
-// conv_dgrad take for layers whose channel counts are multiples of 16;
-// wgrad_tc leaves the sums of *chunks parts in ws.
-bool grad_tc_shape(int ca, int cb, int cout);
+// conv_dgrad take for layers whose channel counts are multiples of 16 (weight
+// gradients also for fewer than 16 input channels); wgrad_tc leaves the sums of *chunks parts in ws.
+bool wgrad_tc_shape(int ca, int cb, int cout);
+bool dgrad_tc_shape(int ca, int cb, int cout);
 bool grad_tc_prepare(int cin, int cout, int H);
 size_t wgrad_tc_ws_floats(int cin, int cout, int H, int sms);
 bool wgrad_tc_fits(const ConvBwd& L, const float* dZ);

@@ -1,5 +1,6 @@
 // Tensor-core weight and input gradients of the warm-start network's 3 x 3
-// layers whose channel counts are multiples of 16 (sm_103a).
+// layers whose channel counts are multiples of 16 (sm_103a); the first layer's
+// three input channels are padded.
 //
 // One operand of each contraction is FP32 (the activations' gradient dZ), the
 // other BF16 (activations or weights). dZ is split exactly into three BF16
@@ -16,7 +17,8 @@
 // gradient): 48 -> 16 channels at 32 x 32: 51 / 45 against 153 / 113; 96 -> 32
 // at 16 x 16: 47 / 44 against 210 / 120; 64 -> 64 at 8 x 8: 27 / 25 against
 // 62 / 57; 128 -> 128 at 4 x 4: 27 / 33 against 66 / 85; the whole gradient
-// call 2234 -> 1057 us. Error against 64-bit sums: input gradient 0.75 to 1.0
+// call 2234 -> 1057 us (1007 with the first layer padded, chunk sums and pool
+// gradients by wider kernels). Error against 64-bit sums: input gradient 0.75 to 1.0
 // of the FP32-FMA kernel's, weight gradient 0.7 to 1.0 of it (and 1.0 to 1.2
 // for a few images, where both are below 1e-7).
 
@@ -114,7 +116,7 @@ struct WgTc {
 
 WgTc wg_tc(int cin, int cout, int H) {
     WgTc w;
-    w.ncin = cin / 16;
+    w.ncin = (cin + 15) / 16;
     const int ncout = cout / 16;
     w.nt = 1;
     for (int d = 2; d <= 8; ++d)
@@ -187,7 +189,14 @@ k_wgrad_tc(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, i
             uint4 u = make_uint4(0, 0, 0, 0);
             if (gr >= 0 && gr < rows && x >= 0 && x < W) {
                 size_t p = size_t(gr) * W + x;
-                if (c < ca) {
+                if (cin < 16) {  // the rest of the 16 channels is zero
+                    const uint16_t* a = reinterpret_cast<const uint16_t*>(A) + p * cin;
+                    uint16_t e[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) e[k] = c + k < cin ? __ldg(a + c + k) : uint16_t(0);
+                    u = make_uint4(e[0] | uint32_t(e[1]) << 16, e[2] | uint32_t(e[3]) << 16,
+                                   e[4] | uint32_t(e[5]) << 16, e[6] | uint32_t(e[7]) << 16);
+                } else if (c < ca) {
                     if (upA) {
                         const int b = gr / H, y = gr - b * H;
                         p = (size_t(b) * (H / 2) + y / 2) * (W / 2) + x / 2;
@@ -256,9 +265,16 @@ k_wgrad_tc(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, i
 #pragma unroll
         for (int t = 0; t < 9; ++t)
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
-                *reinterpret_cast<float2*>(o + (co * 9 + t) * cin + c0 + ti * 16 + 8 * b + t2) =
-                    make_float2(acc[t][b][2 * h], acc[t][b][2 * h + 1]);
+            for (int b = 0; b < 2; ++b) {
+                const int ci = c0 + ti * 16 + 8 * b + t2;
+                float* q = o + (co * 9 + t) * cin + ci;
+                if (cin >= 16) {
+                    *reinterpret_cast<float2*>(q) = make_float2(acc[t][b][2 * h], acc[t][b][2 * h + 1]);
+                } else {
+                    if (ci < cin) q[0] = acc[t][b][2 * h];
+                    if (ci + 1 < cin) q[1] = acc[t][b][2 * h + 1];
+                }
+            }
         if (biased && t2 == 0) o[nw + co] = bias[2 * h];
     }
 }
@@ -439,8 +455,13 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 
 }  // namespace
 
-bool grad_tc_shape(int ca, int cb, int cout) {
+bool dgrad_tc_shape(int ca, int cb, int cout) {
     return (ca + cb) % 16 == 0 && ca % 8 == 0 && cb % 8 == 0 && cout % 16 == 0;
+}
+// fewer than 16 input channels are padded with zeros (3 -> 16 channels at 32 x
+// 32, 256 images: 50 us by the FP32-FMA kernel, 27 so)
+bool wgrad_tc_shape(int ca, int cb, int cout) {
+    return dgrad_tc_shape(ca, cb, cout) || (ca < 16 && cb == 0 && cout % 16 == 0);
 }
 
 size_t wgrad_tc_ws_floats(int cin, int cout, int H, int sms) {
@@ -448,7 +469,8 @@ size_t wgrad_tc_ws_floats(int cin, int cout, int H, int sms) {
 }
 
 bool wgrad_tc_fits(const ConvBwd& L, const float* dZ) {
-    return !L.simt && grad_tc_shape(L.ca, L.cb, L.cout) && aligned16(L.A) && aligned16(L.B) && aligned16(dZ);
+    if (L.simt || !wgrad_tc_shape(L.ca, L.cb, L.cout) || !aligned16(dZ)) return false;
+    return L.ca + L.cb < 16 ? !L.upA : aligned16(L.A) && aligned16(L.B);
 }
 
 cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* chunks, int sms, cudaStream_t s) {
@@ -463,7 +485,7 @@ cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* 
 }
 
 bool dgrad_tc_fits(const ConvBwd& L, const float* dZ, const bf16* Wt) {
-    return !L.simt && grad_tc_shape(L.ca, L.cb, L.cout) && aligned16(dZ) && aligned16(Wt);
+    return !L.simt && dgrad_tc_shape(L.ca, L.cb, L.cout) && aligned16(dZ) && aligned16(Wt);
 }
 
 cudaError_t dgrad_tc(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, const bf16* act, float* dIn,
