@@ -575,14 +575,14 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     } else if (p->N >= 256) {
         if (ext_out || !phase) return FWR_ERR_UNSUPPORTED;
         e = fwr::launch_slab(p->N, k, p->d_scratch, p->d_counters, p->scratch_ctas, static_cast<cudaStream_t>(stream));
-    } else if (p->N == 128 && phase && !ext_out && p->ctas == 0 && fwr::fused_supported(128, 4, p->n) &&
+    } else if (p->N == 128 && phase && !ext_out && p->ctas == 0 && fwr::fused_fits(128, 4, p->n) &&
                fwr::cluster128_wanted(n_frames, p->sms)) {
         // few frames on every SM (no FWR_OPT_CTAS); pupils that the fused kernel
         // takes, whose bits these are
         e = fwr::launch_cluster_f32(k, p->sms, static_cast<cudaStream_t>(stream));
     } else {
-        e = fwr::fused_supported(p->N, 4, p->n) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
-                                                : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
+        e = fwr::fused_fits(p->N, 4, p->n) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
+                                           : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
     }
     return e == cudaSuccess ? FWR_OK : cuda_fail(e, "gerchberg launch");
 }

@@ -14,13 +14,15 @@ namespace fwr {
 #include "fwr_fft.cuh"
 #include "fwr_fused.cuh"
 
+// FP32 on 128^2 (one CTA per SM): the LSQ coefficients live in tensor memory
+template <typename T, int N> __host__ __device__ constexpr bool fused_tmc() { return sizeof(T) == 4 && N == 128; }
+
 // HUD: the Hudgin extension as the initial extension (a separate
 // instantiation, so that the default one carries none of its code)
 template <typename T, int N, bool HUD>
 __global__ void __launch_bounds__(4 * N)
 fused_kernel(Params<T> p) {
-    // FP32 on 128^2 (one CTA per SM): the LSQ coefficients live in tensor memory
-    constexpr bool TMC = sizeof(T) == 4 && N == 128;
+    constexpr bool TMC = fused_tmc<T, N>();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_bad;
     __shared__ uint32_t s_tmem;
@@ -211,9 +213,10 @@ cudaError_t launch_shape(const void* kern, size_t smem, int threads, int* sms, i
 template <typename T, int N>
 cudaError_t launch_n(const Params<T>& p0, cudaStream_t s) {
     // keep the final-filter table in shared memory when it still fits
+    typedef Layout<T, N, fused_tmc<T, N>()> L;
     Params<T> p = p0;
-    p.wf_smem = p.shape != 2 && Layout<T, N>::bytes_wf(p.n) <= size_t(227) * 1024 ? 1 : 0;
-    const size_t smem = p.wf_smem ? Layout<T, N>::bytes_wf(p.n) : Layout<T, N>::bytes(p.n);
+    p.wf_smem = p.shape != 2 && L::bytes_wf(p.n) <= size_t(227) * 1024 ? 1 : 0;
+    const size_t smem = p.wf_smem ? L::bytes_wf(p.n) : L::bytes(p.n);
     auto kern = p.hud ? fused_kernel<T, N, true> : fused_kernel<T, N, false>;
     int sms = 0, per_sm = 0;
     cudaError_t e = launch_shape(reinterpret_cast<const void*>(kern), smem, 4 * N, &sms, &per_sm);
@@ -266,6 +269,11 @@ cudaError_t launch_fft2_f32(int N, const float2* in, float2* out, int F, int inv
 bool fused_supported(int N, int elem_bytes, int n) {
     const size_t b = fused_bytes(N, elem_bytes, n);
     return b != 0 && b <= size_t(227) * 1024;
+}
+
+bool fused_fits(int N, int elem_bytes, int n) {
+    if (N == 128 && elem_bytes == 4) return Layout<float, 128, true>::bytes(n) <= size_t(227) * 1024;
+    return fused_supported(N, elem_bytes, n);
 }
 
 cudaError_t launch_fused_f32(int N, const Params<float>& p, cudaStream_t s) {

@@ -56,7 +56,11 @@ __device__ __forceinline__ void row_role(int tid, int& r, int& n2) {
     n2 = (tid & 1) + 2 * ((tid >> 1) / N);
 }
 
-template <typename T, int N>
+// Shared-memory layout. TMC (coefficients in tensor memory): the 1/|G|^2
+// table is needed during the set-up only and lies in the grid's space; the
+// 33 KB hold the slopes of pupils up to 100 lenslets across (82 otherwise) or
+// the final filter's table.
+template <typename T, int N, bool TMC = false>
 struct Layout {
     typedef typename cvec<T>::type V;
     static constexpr int R = N / 4, H = N / 2, S = N + 2;
@@ -67,8 +71,9 @@ struct Layout {
     static constexpr size_t a = tw2 + size_t(3 * R) * sizeof(V);
     static constexpr size_t t = a + size_t(N) * sizeof(V);
     static constexpr size_t pt = t + size_t(N) * sizeof(V);
-    static constexpr size_t iota = pt + size_t(4 * N) * sizeof(T);
-    static constexpr size_t s0 = (iota + size_t(H + 1) * N * sizeof(T) + 15) & ~size_t(15);
+    static constexpr size_t iota_end = pt + size_t(4 * N) * sizeof(T) + (TMC ? 0 : size_t(H + 1) * N * sizeof(T));
+    static constexpr size_t iota = TMC ? z : pt + size_t(4 * N) * sizeof(T);
+    static constexpr size_t s0 = (iota_end + 15) & ~size_t(15);
     __host__ __device__ static size_t bytes(int n) { return s0 + size_t(n) * s0_stride(n) * sizeof(V); }
     // optional resident copy of the final-filter half-table (same order as iota), after s0
     __host__ __device__ static size_t wf(int n) { return (bytes(n) + 15) & ~size_t(15); }
@@ -359,7 +364,7 @@ __device__ __forceinline__ void fused_setup(FusedCtx<T, N>& c, unsigned char* sm
                                             const uint8_t* mask, int n, int off, int mode, bool wf_smem = false,
                                             uint32_t tmem = 0) {
     typedef typename cvec<T>::type V;
-    typedef Layout<T, N> L;
+    typedef Layout<T, N, TMC> L;
     constexpr int R = N / 4, NT = 4 * N, H = N / 2, S = L::S;
     V* Z = c.Z = reinterpret_cast<V*>(smem + L::z);
     c.xpart = reinterpret_cast<T*>(smem + L::xpart);

@@ -133,9 +133,14 @@ cudaError_t launch_ragged(const RaggedParams& p, int grid, size_t smem, cudaStre
 cudaError_t launch_anygrid_f32(int N, const Params<float>& p, cudaStream_t s);
 cudaError_t launch_anygrid_f64(int N, const Params<double>& p, cudaStream_t s);
 
-// Main fused kernel (fwr_fused.cu). fused_supported() says whether its
-// shared-memory layout fits grid N with n lenslets for the element size.
+// Main fused kernel (fwr_fused.cu). fused_supported() says whether all of its
+// tables fit shared memory on grid N with n lenslets for the element size (what
+// the Hudgin extension, warm starts in BF16 and ragged batches ask for);
+// fused_fits() whether it runs: FP32 on 128^2 keeps one table in tensor memory
+// instead, so 83 to 100 lenslets across run too (1000 frames of 100 x 100, k =
+// 10: 1715 us by the basic kernel, 813 here; one frame 242 and 46).
 bool fused_supported(int N, int elem_bytes, int n);
+bool fused_fits(int N, int elem_bytes, int n);
 cudaError_t launch_fused_f32(int N, const Params<float>& p, cudaStream_t s);
 cudaError_t launch_fused_f64(int N, const Params<double>& p, cudaStream_t s);
 

@@ -3,7 +3,9 @@ one-CTA kernel's phase (kept by an explicit persistent-grid size)."""
 
 import pytest
 
+import oracle
 from paper_1705_04298_gb300 import synth
+from parity_check import FP32_RMS, within
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -85,3 +87,34 @@ def test_cluster_reports_nonfinite_slopes(fwr):
     plan.reconstruct(s, 1)
     assert plan.status() == "FWR_ERR_NONFINITE"
     assert plan.status() == "FWR_OK"
+
+
+@pytest.mark.parametrize("n", [82, 83, 98, 99, 100, 101, 126])
+def test_largest_pupils(fwr, n):
+    """Pupils around the limits of the fused kernel's shared memory (82 with all
+    tables, 100 with the coefficients in tensor memory): one frame by the
+    cluster kernel and many by the fused one with the same bits up to 100, the
+    basic kernel beyond; against the FP64 oracle; the extended slopes; and what
+    needs all tables stays refused."""
+    F = torch.cuda.get_device_properties(0).multi_processor_count + 5
+    s, mask = frames(n, F, n)
+    plan = fwr.Plan(mask, 1.0, fwr.WIENER, 0.01, 0.6, 100.0, grid=128)
+    many = plan.reconstruct(s, 2)
+    ext = torch.empty((2, 2, 128, 128), device="cuda")
+    two = plan.reconstruct(s[:2].contiguous(), 2, ext_out=ext)
+    one = plan.reconstruct(s[:1].contiguous(), 2)
+    assert plan.status() == "FWR_OK"
+    if n <= 100:
+        assert torch.equal(one[0], many[0])
+    for f in range(2):
+        ref, ref_ext = oracle.reconstruct(s[f].cpu().double().numpy(), mask, 1.0, 2, oracle.FILTER_WIENER, 0.01, 0.6,
+                                          100.0, N=128)
+        for got in (many[f], two[f]) if f else (many[f], two[f], one[0]):
+            assert within(got.cpu().numpy(), ref, FP32_RMS, where="n=%d f=%d" % (n, f))
+        assert within(ext[f].cpu().double().numpy(), ref_ext, 10 * FP32_RMS, where="n=%d ext" % n)
+    plan.set_extension(fwr.EXT_HUDGIN)
+    if n <= 82:
+        plan.reconstruct(s[:1].contiguous(), 1)
+    else:
+        with pytest.raises(fwr.FwrError, match="UNSUPPORTED"):
+            plan.reconstruct(s[:1].contiguous(), 1)
