@@ -690,7 +690,7 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
     for (const Layer& L : n->layers) {
         if (L.k != 3) continue;
         gws = std::max(gws, wgrad_ws_floats(L.ca + L.cb, L.cout, L.H, n->sms));
-        if (e == cudaSuccess && !netgrad_prepare(L.ca, L.cb, L.cout, L.H)) e = cudaErrorInvalidValue;
+        if (e == cudaSuccess && !netgrad_fits(L.ca, L.cb, L.cout, L.H)) e = cudaErrorInvalidValue;
     }
     if (e == cudaSuccess) e = cudaMalloc(&n->gws, gws * sizeof(float));
     falloc(&n->dpool, B * 16 * 16 * w1 + B * 8 * 8 * w2 + B * 4 * 4 * w3);

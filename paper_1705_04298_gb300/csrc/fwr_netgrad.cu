@@ -610,6 +610,12 @@ k_out_bwd(const float2* __restrict__ pred, const float2* __restrict__ T, const f
     }
 }
 
+// the limit is set at the launch: a network that is never trained loads no
+// kernel of the backward pass
+template <typename K> cudaError_t set_smem(K kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
+
 int out_ctas(int sms) { return 4 * sms; }
 
 }  // namespace
@@ -630,6 +636,8 @@ cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, flo
     const WgradShape w = wgrad_shape(cin, L.cout, L.H);
     const int rc = wgrad_rows(w, rows, sms), chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad3<32> : L.H == 16 ? k_wgrad3<16> : L.H == 8 ? k_wgrad3<8> : k_wgrad3<4>;
+    const cudaError_t e = set_smem(kern, w.smem);
+    if (e != cudaSuccess) return e;
     kern<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                        ws);
     return reduce_chunks(ws, chunks, n, g, nullptr, sms, s);
@@ -641,6 +649,8 @@ cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn
     const int pairs = Bn * (L.H / 2);
     const DgradShape d = dgrad_shape(L.ca + L.cb, L.H, pairs, sms);
     auto kern = L.H == 32 ? k_dgrad3<32> : L.H == 16 ? k_dgrad3<16> : L.H == 8 ? k_dgrad3<8> : k_dgrad3<4>;
+    const cudaError_t e = set_smem(kern, d.smem);
+    if (e != cudaSuccess) return e;
     kern<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.threads, d.smem, s>>>(dZ, L.cout, Wt, L.ca, L.cb, pairs, d,
                                                                                act, dIn, lo, lo_act);
     return cudaGetLastError();
@@ -658,17 +668,11 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
     return reduce_chunks(ws, used, n, g, loss, sms, s);
 }
 
-bool netgrad_prepare(int ca, int cb, int cout, int H) {
-    const int lim = 227 * 1024, cin = ca + cb;
+bool netgrad_fits(int ca, int cb, int cout, int H) {
+    const int cin = ca + cb;
     if (H != 32 && H != 16 && H != 8 && H != 4) return false;
-    if ((wgrad_tc_shape(ca, cb, cout) || dgrad_tc_shape(ca, cb, cout)) && !grad_tc_prepare(cin, cout, H)) return false;
-    if (std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H, 1ll << 40, 1).smem) > size_t(lim)) return false;
-    cudaError_t e = cudaSuccess;
-    for (auto k : {k_wgrad3<32>, k_wgrad3<16>, k_wgrad3<8>, k_wgrad3<4>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    for (auto k : {k_dgrad3<32>, k_dgrad3<16>, k_dgrad3<8>, k_dgrad3<4>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    return e == cudaSuccess;
+    if ((wgrad_tc_shape(ca, cb, cout) || dgrad_tc_shape(ca, cb, cout)) && !grad_tc_fits(cin, cout, H)) return false;
+    return std::max(wgrad_shape(cin, cout, H).smem, dgrad_shape(cin, H, 1ll << 40, 1).smem) <= size_t(227) * 1024;
 }
 
 }  // namespace net

@@ -38,7 +38,7 @@ cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn
 // gradients also for fewer than 16 input channels); wgrad_tc leaves the sums of *chunks parts in ws.
 bool wgrad_tc_shape(int ca, int cb, int cout);
 bool dgrad_tc_shape(int ca, int cb, int cout);
-bool grad_tc_prepare(int cin, int cout, int H);
+bool grad_tc_fits(int cin, int cout, int H);
 size_t wgrad_tc_ws_floats(int cin, int cout, int H, int sms);
 bool wgrad_tc_fits(const ConvBwd& L, const float* dZ);
 cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* chunks, int sms, cudaStream_t s);
@@ -54,8 +54,8 @@ cudaError_t out_backward(const float* pred, const float* T, const float* LM, con
                          cudaStream_t s);
 size_t out_ws_floats(int C, int sms);
 
-// shared-memory limits of the kernels above for a layer; false if it cannot run
-bool netgrad_prepare(int ca, int cb, int cout, int H);
+// whether the kernels above can run a layer (shared memory)
+bool netgrad_fits(int ca, int cb, int cout, int H);
 
 }  // namespace net
 }  // namespace fwr

@@ -451,6 +451,11 @@ typedef void (*DgKernel)(const float*, int, const bf16*, int, int, int, int, DgT
 DgKernel dg_kernel(int nw) {
     return nw == 4 ? k_dgrad_tc<4> : nw == 3 ? k_dgrad_tc<3> : nw == 2 ? k_dgrad_tc<2> : k_dgrad_tc<1>;
 }
+// the limit is set at the launch: a network that is never trained loads no
+// kernel of the backward pass
+template <typename K> cudaError_t set_smem(K kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -479,6 +484,8 @@ cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* 
     const int rc = wg_tc_rows(w, rows, sms);
     *chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad_tc<32> : L.H == 16 ? k_wgrad_tc<16> : L.H == 8 ? k_wgrad_tc<8> : k_wgrad_tc<4>;
+    const cudaError_t e = set_smem(kern, w.smem);
+    if (e != cudaSuccess) return e;
     kern<<<dim3(*chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                         ws);
     return cudaGetLastError();
@@ -492,20 +499,15 @@ cudaError_t dgrad_tc(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, 
                      float* lo, const bf16* lo_act, int sms, cudaStream_t s) {
     const int pairs = Bn * (L.H / 2);
     const DgTc d = dg_tc(L.ca + L.cb, L.H, pairs, sms);
+    const cudaError_t e = set_smem(dg_kernel(d.nw), d.smem);
+    if (e != cudaSuccess) return e;
     dg_kernel(d.nw)<<<dim3((pairs + d.pairs - 1) / d.pairs, (L.ca + L.cb) / (16 * d.nw)), 32 * d.warps * d.S, d.smem, s>>>(
         dZ, L.cout, Wt, L.ca, L.cb, L.H, pairs, d, act, dIn, lo, lo_act);
     return cudaGetLastError();
 }
 
-bool grad_tc_prepare(int cin, int cout, int H) {
-    const int lim = 227 * 1024;
-    if (std::max(wg_tc(cin, cout, H).smem, dg_tc(cin, H, 1ll << 40, 1).smem) > size_t(lim)) return false;
-    cudaError_t e = cudaSuccess;
-    for (auto k : {k_wgrad_tc<32>, k_wgrad_tc<16>, k_wgrad_tc<8>, k_wgrad_tc<4>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    for (int nw = 1; nw <= 4; ++nw)
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(dg_kernel(nw), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    return e == cudaSuccess;
+bool grad_tc_fits(int cin, int cout, int H) {
+    return std::max(wg_tc(cin, cout, H).smem, dg_tc(cin, H, 1ll << 40, 1).smem) <= size_t(227) * 1024;
 }
 
 }  // namespace net
