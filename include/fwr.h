@@ -140,8 +140,8 @@ typedef enum {
  * with more, a Gerchberg loop started from it. Computed inside the kernels
  * from the staged slopes (no extra memory traffic). Supported by the FFT
  * paths of fwr_reconstruct_ex / fwr_reconstruct_f64 / fwr_reconstruct_host /
- * fwr_reconstruct_static; the DFT-as-GEMM transform and the generic kernel
- * for large pupils on 128x128 grids return FWR_ERR_UNSUPPORTED; batches and
+ * fwr_reconstruct_static; the DFT-as-GEMM transform and large pupils (more
+ * than 82 lenslets across) on 128x128 grids return FWR_ERR_UNSUPPORTED; batches and
  * warm-start objects start from their own extension.
  */
 #define FWR_OPT_EXTENSION 5
@@ -157,7 +157,12 @@ typedef enum {
  *     are kept in shared memory where they fit (1, the default 0) or read from
  *     L2 (2). Values 0..2.
  *   FWR_OPT_CTAS: persistent CTAs of one launch, 0 (default) = every SM times
- *     the CTAs that fit on one; a larger value is clamped to that.
+ *     the CTAs that fit on one; a larger value is clamped to that. With 0 a
+ *     launch of few frames on 128x128 or larger grids puts several SMs on a
+ *     frame (128x128: a cluster of CTAs; 256x256 and 512x512: a cooperative
+ *     launch, whose CTAs must all be resident); any other value keeps one CTA
+ *     per frame. (The FP64 entry point does the same on 32x32 and 64x64, where
+ *     the two agree to rounding.)
  */
 #define FWR_OPT_SHAPE 6
 #define FWR_OPT_CTAS 7
