@@ -10,7 +10,7 @@
 // operands come from shared memory in 16-byte loads, few loads per FMA.
 // Measured on 256 images at width 16, the whole gradient call: 90.6 ms with
 // scalar kernels (one block per output channel and tap, operands from global
-// memory), 2.5 ms with these, 1.01 ms with the tensor cores'.
+// memory), 2.5 ms with these, 0.96 ms with the tensor cores'.
 
 #include <stdint.h>
 

@@ -17,8 +17,9 @@
 // gradient): 48 -> 16 channels at 32 x 32: 51 / 45 against 153 / 113; 96 -> 32
 // at 16 x 16: 47 / 44 against 210 / 120; 64 -> 64 at 8 x 8: 27 / 25 against
 // 62 / 57; 128 -> 128 at 4 x 4: 27 / 33 against 66 / 85; the whole gradient
-// call 2234 -> 1057 us (1007 with the first layer padded, chunk sums and pool
-// gradients by wider kernels). Error against 64-bit sums: input gradient 0.75 to 1.0
+// call 2234 -> 1057 us (1004 with the first layer padded, chunk sums and pool
+// gradients by wider kernels; 961 with the weight gradient's input rows copied
+// asynchronously). Error against 64-bit sums: input gradient 0.75 to 1.0
 // of the FP32-FMA kernel's, weight gradient 0.7 to 1.0 of it (and 1.0 to 1.2
 // for a few images, where both are below 1e-7).
 
@@ -64,6 +65,13 @@ __device__ __forceinline__ void mma3(float (&acc)[4], const uint32_t (&a)[3][4],
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] += t[i];
 }
+
+// asynchronous 16-byte copy global -> shared; zeros when !ok (src is not read)
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // the three BF16 parts of x and y, packed (x in the lower half); an infinity
 // stays in the first part
@@ -186,27 +194,25 @@ k_wgrad_tc(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, i
         for (int i = tid; i < (nr + 2) * (W + 2) * 2 * w.nt; i += blockDim.x) {
             const int q = div_by(i, w.by_in), v = i - q * 2 * w.nt, xx = q % (W + 2), r = q / (W + 2);
             const int gr = r0 - 1 + r, x = xx - 1, c = c0 + 8 * v;
-            uint4 u = make_uint4(0, 0, 0, 0);
-            if (gr >= 0 && gr < rows && x >= 0 && x < W) {
-                size_t p = size_t(gr) * W + x;
-                if (cin < 16) {  // the rest of the 16 channels is zero
-                    const uint16_t* a = reinterpret_cast<const uint16_t*>(A) + p * cin;
-                    uint16_t e[8];
+            const bool ok = gr >= 0 && gr < rows && x >= 0 && x < W;
+            unsigned char* const dst = in + q * w.pin + 16 * v;
+            size_t p = ok ? size_t(gr) * W + x : 0;
+            if (cin < 16) {  // the rest of the 16 channels is zero
+                const uint16_t* a = reinterpret_cast<const uint16_t*>(A) + p * cin;
+                uint16_t e[8];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) e[k] = c + k < cin ? __ldg(a + c + k) : uint16_t(0);
-                    u = make_uint4(e[0] | uint32_t(e[1]) << 16, e[2] | uint32_t(e[3]) << 16,
-                                   e[4] | uint32_t(e[5]) << 16, e[6] | uint32_t(e[7]) << 16);
-                } else if (c < ca) {
-                    if (upA) {
-                        const int b = gr / H, y = gr - b * H;
-                        p = (size_t(b) * (H / 2) + y / 2) * (W / 2) + x / 2;
-                    }
-                    u = __ldg(reinterpret_cast<const uint4*>(A + p * ca + c));
-                } else {
-                    u = __ldg(reinterpret_cast<const uint4*>(Bt + p * cb + (c - ca)));
+                for (int k = 0; k < 8; ++k) e[k] = ok && c + k < cin ? __ldg(a + c + k) : uint16_t(0);
+                *reinterpret_cast<uint4*>(dst) = make_uint4(e[0] | uint32_t(e[1]) << 16, e[2] | uint32_t(e[3]) << 16,
+                                                            e[4] | uint32_t(e[5]) << 16, e[6] | uint32_t(e[7]) << 16);
+            } else if (c < ca) {
+                if (upA) {
+                    const int b = gr / H, y = gr - b * H;
+                    p = ok ? (size_t(b) * (H / 2) + y / 2) * (W / 2) + x / 2 : 0;
                 }
+                cp16(dst, A + p * ca + c, ok);
+            } else {
+                cp16(dst, Bt + p * cb + (c - ca), ok);
             }
-            *reinterpret_cast<uint4*>(in + q * w.pin + 16 * v) = u;
         }
 #pragma unroll 4
         for (int i = tid; i < nr * W * 4 * w.mt; i += blockDim.x) {
@@ -214,6 +220,7 @@ k_wgrad_tc(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, i
             const float4 v = __ldg(reinterpret_cast<const float4*>(dZ + (size_t(r0) * W + q) * cout + m0) + c);
             store_split(zp + q * w.pz + 8 * c, plane, v);
         }
+        cp_wait();
         __syncthreads();
         for (int ch = s; ch < nr * W / 16; ch += w.S) {
             uint32_t a[3][4];
