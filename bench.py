@@ -97,9 +97,10 @@ TRAFFIC = {
     # the launcher caches its occupancy queries (kernel unchanged; ncu --metrics
     # dram__bytes_read.sum,dram__bytes_write.sum, bench.py --workload fused128): 13.636 MB + 6.874 MB
     "87a73a622d7087ed": 20509952,
-    # twiddles and final filter written out, the 1/|G|^2 table in the grid's space (ncu --metrics
-    # dram__bytes_read.sum,dram__bytes_write.sum, bench.py --workload fused128): 13.647 MB + 6.858 MB
-    "6ee30c3d65a48566": 20504832,
+    # twiddles and final filter written out, the 1/|G|^2 table in the grid's space, the next frame's
+    # warm start prefetched (ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, bench.py
+    # --workload fused128): 13.010 MB + 5.920 MB
+    "d710ab45b3e80914": 18929408,
 }
 
 
