@@ -90,11 +90,14 @@ template <int N> struct SlabLayout {
     static constexpr size_t tw = lb + LB_BYTES;             // N cells: w_N^j
     static constexpr size_t a = tw + size_t(N) * 8;         // N cells: a(u)
     static constexpr size_t t = a + size_t(N) * 8;          // N cells: T(u)
-    // w_N^(n2 k1) at [k1][n2], 16 x RB and RB x 16 cells (256^2: the same table)
+    // w_N^(n2 k1) at [k1][n2], 16 x RB and RB x 16 cells (256^2: the same
+    // table, and the groups' fill spectra in the place of the second)
     static constexpr size_t twa = t + size_t(N) * 8;
-    static constexpr size_t twi = N == 256 ? twa : twa + size_t(16) * RB * 8;
-    static constexpr size_t eys = twi + size_t(RB) * 16 * 8;  // 256^2: the groups' fill spectra
-    static constexpr size_t pt = eys + (N == 256 ? size_t(2) * (S2::SC + 1) * 8 : 0);  // 4 N floats
+    static constexpr size_t eys = twa + size_t(16) * RB * 8;
+    static constexpr size_t twi = N == 256 ? twa : eys;
+    static constexpr size_t pt = eys + size_t(RB) * 16 * 8;  // 4 N floats
+    static_assert(N != 256 || 2 * (S2::SC + 1) * 8 <= RB * 16 * 8, "fill spectra fit");
+    static_assert(N != 256 || (S1::SC + 1) * 8 <= RB * 16 * 8, "fill spectra fit");
     static constexpr size_t WTS = 2 * size_t(S2::WS) * N > size_t(S1::WS) * N ? 2 * size_t(S2::WS) * N
                                                                                : size_t(S1::WS) * N;
     static constexpr size_t wts = pt + size_t(4) * N * 4;

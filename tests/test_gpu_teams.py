@@ -96,3 +96,15 @@ def test_256_every_bin(fwr, n, k, periodic, shape):
     ref, _ = oracle.reconstruct(s[0].cpu().double().numpy(), mask, 1.0, k, oracle.FILTER_WIENER, 0.01, 0.6, 100.0, periodic,
                                 ext_init=ext[0].astype(np.float64), N=256)
     assert within(ph[0].cpu().numpy(), ref, FP32_RMS, where="n=%d" % n)
+
+
+def test_256_largest_pupil(fwr):
+    """209 lenslets across are the most that 256^2 takes; the largest runs."""
+    with pytest.raises(fwr.FwrError, match="UNSUPPORTED"):
+        fwr.Plan(synth.pupil_mask(210), 1.0, fwr.WIENER, 0.01, 0.6, 100.0, grid=256)
+    s, mask = frames(209, 1, 5)
+    plan = fwr.Plan(mask, 1.0, fwr.WIENER, 0.01, 0.6, 100.0, grid=256)
+    ph = plan.reconstruct(s, 1)
+    ref, _ = oracle.reconstruct(s[0].cpu().double().numpy(), mask, 1.0, 1, oracle.FILTER_WIENER, 0.01, 0.6, 100.0,
+                                N=256)
+    assert within(ph[0].cpu().numpy(), ref, FP32_RMS, where="n=209")
