@@ -66,7 +66,8 @@ template <int N, int GROUPS> struct SlabShape {
     static constexpr int SL = (N == 256 ? 64 : 32) / GROUPS;  // lines per slab
     static constexpr int SGT = SNT / GROUPS;                // threads per group
     static constexpr int SC = SL / 2;                       // first-half columns of a column slab
-    static constexpr int WS = SC + 1;                       // row stride of a group's spectral weights
+    static constexpr int WS = SC + 1;                       // row stride of a group's spectral weights (512^2)
+    static constexpr int WP = SC + 4;                       // 256^2: rows 0 .. N/2 only, 16-byte aligned
     static constexpr int CLS = N + 1;                       // column phase: line stride (cells)
     // row phase: a line's groups of 16, stride 17 (inverse), or of RB, stride
     // RB + 1 (forward), in the same cells
@@ -160,6 +161,10 @@ __device__ __forceinline__ void team_leave(const TeamBar& b) {
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // prefetch [p, p + bytes) into L2, one 128-byte line per thread (of nthreads) and step
@@ -323,7 +328,7 @@ __device__ __forceinline__ void fill_pair(float2& z1, float2& z2, float2 ey, flo
 template <int GROUPS>
 __device__ __forceinline__ void column_spectrum(const SlabCtx& c, int s, int g, int tg, bool fill, bool final) {
     typedef SlabShape<256, GROUPS> Sh;
-    constexpr int N = 256, SC = Sh::SC, WS = Sh::WS, CLS = Sh::CLS, SGT = Sh::SGT;
+    constexpr int N = 256, SC = Sh::SC, WS = Sh::WS, WP = Sh::WP, CLS = Sh::CLS, SGT = Sh::SGT;
     float2* const Lb = c.Lb + g * Sh::LB_CELLS;
     const float* const wts = c.wts + g * WS * N;
     float2* const eys = c.eys + g * WS;
@@ -396,10 +401,10 @@ __device__ __forceinline__ void column_spectrum(const SlabCtx& c, int s, int g, 
                 float4 p0 = pt[0], pm = pt[N / 2];
                 const float4 r0 = p0, rm = pm;
                 p0.z *= 0.5f, p0.w *= 0.5f, pm.z *= 0.5f, pm.w *= 0.5f;
-                lsq_pair(m0, d0, p0, rm, wts[(N / 2) * WS]);
+                lsq_pair(m0, d0, p0, rm, wts[(N / 2) * WP]);
                 lsq_pair(m1, d1, pm, r0, wts[SC]);
             } else {
-                final_pair(m0, d0, cmul_rn(c.A[0], c.Tt[N / 2]), cmul_rn(c.Tt[0], c.A[N / 2]), wts[(N / 2) * WS]);
+                final_pair(m0, d0, cmul_rn(c.A[0], c.Tt[N / 2]), cmul_rn(c.Tt[0], c.A[N / 2]), wts[(N / 2) * WP]);
                 final_pair(m1, d1, cmul_rn(c.A[N / 2], c.Tt[0]), cmul_rn(c.Tt[N / 2], c.A[0]), wts[SC]);
             }
         }
@@ -416,7 +421,7 @@ __device__ __forceinline__ void column_spectrum(const SlabCtx& c, int s, int g, 
             for (int k2 = 8 * h; k2 < 8 * h + 8; ++k2) {
                 const int ky = q + 16 * k2;
                 fill_pair(y[0][k2], y[1][15 - k2], ey, c.tw[ky]);
-                lsq_pair(y[0][k2], y[1][15 - k2], pu, pt[ky], wts[ky * WS + col]);
+                lsq_pair(y[0][k2], y[1][15 - k2], pu, pt[ky], wts[(h ? N - ky : ky) * WP + col]);
             }
         }
     } else {
@@ -428,7 +433,8 @@ __device__ __forceinline__ void column_spectrum(const SlabCtx& c, int s, int g, 
             for (int k2 = 8 * h; k2 < 8 * h + 8; ++k2) {
                 const int ky = q + 16 * k2;
                 fill_pair(y[0][k2], y[1][15 - k2], ey, c.tw[ky]);
-                final_pair(y[0][k2], y[1][15 - k2], cmul_rn(Akx, c.Tt[ky]), cmul_rn(Tkx, c.A[ky]), wts[ky * WS + col]);
+                final_pair(y[0][k2], y[1][15 - k2], cmul_rn(Akx, c.Tt[ky]), cmul_rn(Tkx, c.A[ky]),
+                           wts[(h ? N - ky : ky) * WP + col]);
             }
         }
     }
@@ -529,10 +535,19 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
             for (int s = s0; s < N / SL; s += ds) {
                 const int kx = slab_col<N, SC>(s, cl);
                 const int pl = partner_line<SC>(s, cl);
-                {
+                const float* wt = final ? tab.wfin : tab.iota;
+                if constexpr (PAIRED) {
+                    // spectral weights of the first-half columns (even in ky): rows
+                    // 0 .. N/2 of the half-table
+                    for (int k = tg; k < (H + 1) * (SC / 4); k += SGT) {
+                        const int row = k / (SC / 4), j = 4 * (k % (SC / 4));
+                        cp_async16(wts + row * Sh::WP + j, wt + row * N + SC * s + j);
+                    }
+                    if (s == 0)  // line SC: the self-paired column N/2
+                        for (int k = tg; k <= H; k += SGT) cp_async4(wts + k * Sh::WP + SC, wt + k * N + H);
+                } else {
                     // spectral weights of the first-half columns: wts[ky][j] at
                     // (ky, kx) from the half-table (rows 0..N/2; (-ky, -kx) beyond)
-                    const float* wt = final ? tab.wfin : tab.iota;
                     const int j = tg % SC, kxj = slab_col<N, SC>(s, j), kxn = (N - kxj) & (N - 1);
                     for (int k = tg / SC; k < N; k += SGT / SC)
                         cp_async4(wts + k * WS + j, wt + (k <= H ? k * N + kxj : (N - k) * N + kxn));
