@@ -66,8 +66,9 @@ template <int N, int GROUPS> struct SlabShape {
     static constexpr int SL = (N == 256 ? 64 : 32) / GROUPS;  // lines per slab
     static constexpr int SGT = SNT / GROUPS;                // threads per group
     static constexpr int SC = SL / 2;                       // first-half columns of a column slab
-    static constexpr int WS = SC + 1;                       // row stride of a group's spectral weights (512^2)
-    static constexpr int WP = SC + 4;                       // 256^2: rows 0 .. N/2 only, 16-byte aligned
+    static constexpr int WP = SC + 4;                       // row stride of a group's spectral weights (rows 0 .. N/2)
+    static constexpr int WS = SC + 1;                       // N WS values are set aside for them
+    static_assert((N / 2 + 1) * WP <= N * WS && WP % 4 == 0 && (N * WS) % 4 == 0, "weights fit, 16-byte aligned");
     static constexpr int CLS = N + 1;                       // column phase: line stride (cells)
     // row phase: a line's groups of 16, stride 17 (inverse), or of RB, stride
     // RB + 1 (forward), in the same cells
@@ -499,7 +500,7 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                                            const float* ext, float* phase, int iters, float2* G,
                                            const int16_t* hud = nullptr, int rank = 0, TeamBar* bar = nullptr) {
     typedef SlabShape<N, GROUPS> Sh;
-    constexpr int SL = Sh::SL, SGT = Sh::SGT, SC = Sh::SC, WS = Sh::WS, RB = Sh::RB, H = Sh::H;
+    constexpr int SL = Sh::SL, SGT = Sh::SGT, SC = Sh::SC, WS = Sh::WS, WP = Sh::WP, RB = Sh::RB, H = Sh::H;
     constexpr int CLS = Sh::CLS, RLS = Sh::RLS, NA = Sh::NA, NB = Sh::NB;
     const int g = threadIdx.x / SGT, tg = threadIdx.x % SGT;
     // first slab and step of this group
@@ -535,26 +536,15 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
             for (int s = s0; s < N / SL; s += ds) {
                 const int kx = slab_col<N, SC>(s, cl);
                 const int pl = partner_line<SC>(s, cl);
+                // spectral weights of the first-half columns (even in ky): rows
+                // 0 .. N/2 of the half-table
                 const float* wt = final ? tab.wfin : tab.iota;
-                if constexpr (PAIRED) {
-                    // spectral weights of the first-half columns (even in ky): rows
-                    // 0 .. N/2 of the half-table
-                    for (int k = tg; k < (H + 1) * (SC / 4); k += SGT) {
-                        const int row = k / (SC / 4), j = 4 * (k % (SC / 4));
-                        cp_async16(wts + row * Sh::WP + j, wt + row * N + SC * s + j);
-                    }
-                    if (s == 0)  // line SC: the self-paired column N/2
-                        for (int k = tg; k <= H; k += SGT) cp_async4(wts + k * Sh::WP + SC, wt + k * N + H);
-                } else {
-                    // spectral weights of the first-half columns: wts[ky][j] at
-                    // (ky, kx) from the half-table (rows 0..N/2; (-ky, -kx) beyond)
-                    const int j = tg % SC, kxj = slab_col<N, SC>(s, j), kxn = (N - kxj) & (N - 1);
-                    for (int k = tg / SC; k < N; k += SGT / SC)
-                        cp_async4(wts + k * WS + j, wt + (k <= H ? k * N + kxj : (N - k) * N + kxn));
-                    if (s == 0)  // line SC: the self-paired column N/2
-                        for (int k = tg; k < N; k += SGT)
-                            cp_async4(wts + k * WS + SC, wt + (k <= H ? k : N - k) * N + H);
+                for (int k = tg; k < (H + 1) * (SC / 4); k += SGT) {
+                    const int row = k / (SC / 4), j = 4 * (k % (SC / 4));
+                    cp_async16(wts + row * WP + j, wt + row * N + SC * s + j);
                 }
+                if (s == 0)  // line SC: the self-paired column N/2
+                    for (int k = tg; k <= H; k += SGT) cp_async4(wts + k * WP + SC, wt + k * N + H);
                 // pass A: 16-point DFTs over rows RB n1 + n2 of the column, from memory
                 {
                     float2 x[NA][16];
@@ -608,8 +598,6 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                     }
                     const float4 pu = *reinterpret_cast<const float4*>(pt + 4 * kx);
                     const float2 Akx = A[kx], Tkx = Tt[kx];
-                    // weight column of this line and whether its rows are mirrored
-                    const bool first = cl < SC || (s == 0 && cl == SC);
                     const int wcol = (s == 0 && cl == SC) ? SC : (cl % SC);
 #pragma unroll
                     for (int i = 0; i < NB; ++i) {
@@ -625,7 +613,7 @@ __device__ __forceinline__ bool slab_frame(const SlabCtx& c, const Tables<float>
                                 z1 = make_float2(z1.x + c0.y, z1.y - c0.x);
                                 z2 = make_float2(z2.x - c0.y, z2.y - c0.x);
                             }
-                            const float w = wts[(first ? ky : kyn) * WS + wcol];
+                            const float w = wts[(k2 < RB / 2 ? ky : N - ky) * WP + wcol];
                             const float4 pv = *reinterpret_cast<const float4*>(pt + 4 * ky);
                             if (!final) {
                                 // Algorithm 1 step 2: Z'(k) = w (a z1 + b conj z2) with, at the
