@@ -169,15 +169,8 @@ cudaError_t launch_fft2_n(const float2* in, float2* out, int F, int inverse, con
 }
 
 // Per (device, kernel, shared-memory size): the SM count and the resident CTAs
-// per SM (these queries were on every call's path). The kernel's
-// shared-memory limit is a property of the function, so it is tracked per
-// (device, kernel) and only ever raised: a smaller launch never lowers it
-// below what a cached larger launch needs.
-struct KernelLimit {
-    int dev;
-    const void* kern;
-    size_t smem_max;
-};
+// per SM (these queries were on every call's path); a size in the cache is
+// within the kernel's limit, which is only ever raised.
 struct LaunchShape {
     int dev;
     const void* kern;
@@ -187,24 +180,11 @@ struct LaunchShape {
 
 cudaError_t launch_shape(const void* kern, size_t smem, int threads, int* sms, int* per_sm) {
     static std::mutex mu;
-    static std::vector<KernelLimit> limits;
     static std::vector<LaunchShape> cache;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(mu);
-    KernelLimit* lim = nullptr;
-    for (KernelLimit& l : limits)
-        if (l.dev == dev && l.kern == kern) lim = &l;
-    if (!lim || lim->smem_max < smem) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess)
-            return e;
-        if (lim) {
-            lim->smem_max = smem;
-        } else {
-            limits.push_back(KernelLimit{dev, kern, smem});
-        }
-    }
     for (const LaunchShape& c : cache)
         if (c.dev == dev && c.kern == kern && c.smem == smem) {
             *sms = c.sms;
@@ -212,6 +192,7 @@ cudaError_t launch_shape(const void* kern, size_t smem, int threads, int* sms, i
             return cudaSuccess;
         }
     LaunchShape c{dev, kern, smem, 0, 0};
+    if ((e = raise_smem_limit(kern, smem)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.per_sm, kern, threads, smem)) != cudaSuccess) return e;
     cache.push_back(c);
@@ -274,6 +255,29 @@ cudaError_t launch_fft2_f32(int N, const float2* in, float2* out, int F, int inv
         case 128: return launch_fft2_n<128>(in, out, F, inverse, tw, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t raise_smem_limit(const void* kern, size_t bytes) {
+    struct Limit {
+        int dev;
+        const void* kern;
+        size_t bytes;
+    };
+    static std::mutex mu;
+    static std::vector<Limit> limits;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    Limit* lim = nullptr;
+    for (Limit& l : limits)
+        if (l.dev == dev && l.kern == kern) lim = &l;
+    if (lim && lim->bytes >= bytes) return cudaSuccess;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes))) != cudaSuccess)
+        return e;
+    if (lim) lim->bytes = bytes;
+    else limits.push_back(Limit{dev, kern, bytes});
+    return cudaSuccess;
 }
 
 bool fused_supported(int N, int elem_bytes, int n) {

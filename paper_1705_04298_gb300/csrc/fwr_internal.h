@@ -62,6 +62,15 @@ template <typename T> struct Params {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// Raise a kernel's dynamic shared-memory limit on the current device to `bytes`
+// where it is lower. The limit belongs to the function on the device, whoever
+// launches it: it is only ever raised, under a lock, so that neither a smaller
+// launch nor another thread's leaves it below what a launch needs.
+cudaError_t raise_smem_limit(const void* kern, size_t bytes);
+template <typename... A> cudaError_t raise_smem_limit(void (*kern)(A...), size_t bytes) {
+    return raise_smem_limit(reinterpret_cast<const void*>(kern), bytes);
+}
+
 // Where Eq. PC is applied (same values as FWR_PERIODIC_* in fwr.h).
 enum : int { PERIODIC_BEFORE_EACH_FFT = 0, PERIODIC_FINAL_ONLY = 1, PERIODIC_NONE = 2 };
 

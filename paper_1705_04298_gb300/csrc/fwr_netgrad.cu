@@ -16,6 +16,7 @@
 
 #include <algorithm>
 
+#include "fwr_internal.h"
 #include "fwr_netgrad.h"
 
 namespace fwr {
@@ -610,12 +611,6 @@ k_out_bwd(const float2* __restrict__ pred, const float2* __restrict__ T, const f
     }
 }
 
-// the limit is set at the launch: a network that is never trained loads no
-// kernel of the backward pass
-template <typename K> cudaError_t set_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-}
-
 int out_ctas(int sms) { return 4 * sms; }
 
 }  // namespace
@@ -636,7 +631,9 @@ cudaError_t conv_wgrad(const ConvBwd& L, const float* dZ, int Bn, float* ws, flo
     const WgradShape w = wgrad_shape(cin, L.cout, L.H);
     const int rc = wgrad_rows(w, rows, sms), chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad3<32> : L.H == 16 ? k_wgrad3<16> : L.H == 8 ? k_wgrad3<8> : k_wgrad3<4>;
-    const cudaError_t e = set_smem(kern, w.smem);
+    // limits are raised at the launches: a network that is never trained loads
+    // no kernel of the backward pass
+    const cudaError_t e = raise_smem_limit(kern, w.smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                        ws);
@@ -649,7 +646,7 @@ cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn
     const int pairs = Bn * (L.H / 2);
     const DgradShape d = dgrad_shape(L.ca + L.cb, L.H, pairs, sms);
     auto kern = L.H == 32 ? k_dgrad3<32> : L.H == 16 ? k_dgrad3<16> : L.H == 8 ? k_dgrad3<8> : k_dgrad3<4>;
-    const cudaError_t e = set_smem(kern, d.smem);
+    const cudaError_t e = raise_smem_limit(kern, d.smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.threads, d.smem, s>>>(dZ, L.cout, Wt, L.ca, L.cb, pairs, d,
                                                                                act, dIn, lo, lo_act);

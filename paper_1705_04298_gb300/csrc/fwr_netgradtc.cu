@@ -27,6 +27,7 @@
 
 #include <algorithm>
 
+#include "fwr_internal.h"
 #include "fwr_netgrad.h"
 
 namespace fwr {
@@ -458,11 +459,6 @@ typedef void (*DgKernel)(const float*, int, const bf16*, int, int, int, int, DgT
 DgKernel dg_kernel(int nw) {
     return nw == 4 ? k_dgrad_tc<4> : nw == 3 ? k_dgrad_tc<3> : nw == 2 ? k_dgrad_tc<2> : k_dgrad_tc<1>;
 }
-// the limit is set at the launch: a network that is never trained loads no
-// kernel of the backward pass
-template <typename K> cudaError_t set_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-}
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -491,7 +487,7 @@ cudaError_t wgrad_tc(const ConvBwd& L, const float* dZ, int Bn, float* ws, int* 
     const int rc = wg_tc_rows(w, rows, sms);
     *chunks = (rows + rc - 1) / rc;
     auto kern = L.H == 32 ? k_wgrad_tc<32> : L.H == 16 ? k_wgrad_tc<16> : L.H == 8 ? k_wgrad_tc<8> : k_wgrad_tc<4>;
-    const cudaError_t e = set_smem(kern, w.smem);
+    const cudaError_t e = raise_smem_limit(kern, w.smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(*chunks, w.ny), w.threads, w.smem, s>>>(dZ, L.cout, L.A, L.ca, L.upA ? 1 : 0, L.B, L.cb, rows, rc, w,
                                                         ws);
@@ -506,7 +502,7 @@ cudaError_t dgrad_tc(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn, 
                      float* lo, const bf16* lo_act, int sms, cudaStream_t s) {
     const int pairs = Bn * (L.H / 2);
     const DgTc d = dg_tc(L.ca + L.cb, L.H, pairs, sms);
-    const cudaError_t e = set_smem(dg_kernel(d.nw), d.smem);
+    const cudaError_t e = raise_smem_limit(dg_kernel(d.nw), d.smem);
     if (e != cudaSuccess) return e;
     dg_kernel(d.nw)<<<dim3((pairs + d.pairs - 1) / d.pairs, (L.ca + L.cb) / (16 * d.nw)), 32 * d.warps * d.S, d.smem, s>>>(
         dZ, L.cout, Wt, L.ca, L.cb, L.H, pairs, d, act, dIn, lo, lo_act);

@@ -1,0 +1,74 @@
+"""A kernel's shared-memory limit belongs to the function on the device, not
+to a plan, batch or network: objects of different sizes that share a kernel
+run in any order and from several threads."""
+
+import threading
+
+import numpy as np
+import pytest
+
+from oracle import unet
+from paper_1705_04298_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fwr():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1705_04298_gb300 import fwr as m
+    m.load()
+    return m
+
+
+def slopes(n, F, seed):
+    mask = synth.pupil_mask(n)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randn((F, 2, n, n), generator=g, device="cuda") * torch.tensor(mask, device="cuda"), mask
+
+
+def at_once(calls, times):
+    """Each of `calls` `times` times in a thread of its own; the first error is raised."""
+    errors = []
+    start = threading.Barrier(len(calls))
+
+    def work(call):
+        try:
+            start.wait()
+            for _ in range(times):
+                call()
+        except Exception as e:  # noqa: BLE001  (re-raised below)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(c,)) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def net_problem(fwr, w, F):
+    n = 40
+    s, mask = slopes(n, F, w)
+    plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=128)
+    net = fwr.Net(w, F, unet.init_params(w, w))
+    return plan, net, s, torch.randn((F, 2, 128, 128), device="cuda")
+
+
+def test_gradients_of_two_networks_from_two_threads(fwr):
+    """The layers of a backward pass need different sizes of one kernel."""
+    runs = []
+    for w in (16, 32):
+        plan, net, s, e = net_problem(fwr, w, 4)
+        runs.append((plan, net, s, e, net.gradients(plan, s, e), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def call(plan, net, s, e, ref, stream):
+        loss, g = net.gradients(plan, s, e, stream=stream)
+        assert loss == ref[0] and np.array_equal(g, ref[1])
+
+    at_once([lambda r=r: call(*r) for r in runs], 300)
