@@ -106,7 +106,7 @@ cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, unsigned
 // The same kernel on the library's static scratch array (no allocation):
 // at most STATIC_SLAB_GRIDS CTAs; cudaErrorInvalidValue for ctas outside
 // 1..STATIC_SLAB_GRIDS. static_slab_prepare (current device) returns the
-// array's device address and sets the kernel's shared-memory limit for n
+// array's device address and raises the kernel's shared-memory limit for n
 // lenslets; launch_slab_static takes that address.
 enum : int { STATIC_SLAB_GRIDS = 16 };
 cudaError_t static_slab_prepare(int n, float2** addr);

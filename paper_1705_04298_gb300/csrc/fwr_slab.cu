@@ -67,11 +67,11 @@ typedef void (*SlabKernel)(Params<float>, float2*);
 typedef void (*SlabTeamKernel)(Params<float>, float2*, unsigned*, int);
 
 // the kernel of grid N and a shape (1 or 2 warp groups; 0 is 2) with its
-// shared-memory limit set for n lenslets
+// shared-memory limit raised for n lenslets
 cudaError_t slab_kernel_for(int N, int shape, int n, SlabKernel* k) {
     if (N == 512) *k = shape == 1 ? slab_kernel<512, 1> : slab_kernel<512, 2>;
     else *k = shape == 1 ? slab_kernel<256, 1> : slab_kernel<256, 2>;
-    return cudaFuncSetAttribute(*k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(slab_layout_bytes_n(N, n)));
+    return raise_smem_limit(*k, slab_layout_bytes_n(N, n));
 }
 
 }  // namespace
@@ -127,7 +127,7 @@ cudaError_t launch_team(int N, int team, const Params<float>& p, float2* scratch
                         cudaStream_t s) {
     const SlabTeamKernel kern = N == 512 ? slab_team_kernel<512> : slab_team_kernel<256>;
     const size_t smem = slab_smem_bytes(N, p.n);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = raise_smem_limit(kern, smem);
     if (e != cudaSuccess) return e;
     int teams = max_ctas / team;
     if (p.F < teams) teams = p.F;
@@ -196,7 +196,7 @@ static __device__ __align__(256) float2 g_static_slab_scratch[STATIC_SLAB_GRIDS 
 
 // Host code cannot use the array's name as a device address: look the address
 // up with the device current (this also loads the module on that device, so a
-// later call does no loading) and set the kernel's shared-memory limit.
+// later call does no loading) and raise the kernel's shared-memory limit.
 cudaError_t static_slab_prepare(int n, float2** addr) {
     void* ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_slab_scratch);

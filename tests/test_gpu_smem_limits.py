@@ -72,3 +72,35 @@ def test_gradients_of_two_networks_from_two_threads(fwr):
         assert loss == ref[0] and np.array_equal(g, ref[1])
 
     at_once([lambda r=r: call(*r) for r in runs], 300)
+
+
+def test_few_frames_of_several_pupils_from_several_threads(fwr):
+    """256^2 plans of different pupils need different sizes of one kernel."""
+    runs = []
+    for n in (205, 70, 40, 180, 30, 100, 60, 50):
+        s, mask = slopes(n, 1, n)
+        plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=256)
+        ref = plan.reconstruct(s, 0).clone()
+        runs.append((plan, s, ref, torch.empty_like(ref), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def call(plan, s, ref, out, stream):
+        plan.reconstruct(s, 0, out, stream=stream)
+        with torch.cuda.stream(stream):
+            assert torch.equal(out, ref)
+
+    at_once([lambda r=r: call(*r) for r in runs], 1500)
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+def test_static_scratch_after_a_smaller_plan(fwr, shape):
+    s, mask = slopes(200, 2, 5)
+    plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=256)
+    plan.set_shape(shape)
+    ref = plan.reconstruct_static(s, 1, ctas=2).clone()
+    small, smask = slopes(60, 2, 6)
+    other = fwr.Plan(smask, 1.0, fwr.LSQ, grid=256)
+    other.set_shape(shape)
+    other.set_ctas(2)
+    other.reconstruct(small, 1)
+    assert torch.equal(plan.reconstruct_static(s, 1, ctas=2), ref)
