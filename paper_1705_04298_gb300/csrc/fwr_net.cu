@@ -716,15 +716,13 @@ fwr_status fwr_net_create(fwr_net** out, int width, int max_batch, const float* 
         tc_smem = 0;
     }
     if (e == cudaSuccess && tc_smem) {
-        const int v = int(tc_smem);
-        e = cudaFuncSetAttribute(k_conv_tc<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+        e = fwr::raise_smem_limit(k_conv_tc<8>, tc_smem);
+        if (e == cudaSuccess) e = fwr::raise_smem_limit(k_conv_tc<4>, tc_smem);
+        if (e == cudaSuccess) e = fwr::raise_smem_limit(k_conv_tc<2>, tc_smem);
+        if (e == cudaSuccess) e = fwr::raise_smem_limit(k_conv_tc<1>, tc_smem);
     }
     if (e == cudaSuccess) e = unet_forward_prepare();
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_conv_fwd<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fwd_smem));
+    if (e == cudaSuccess) e = fwr::raise_smem_limit(k_conv_fwd<3>, fwd_smem);
     if (e != cudaSuccess) {
         free_net(n);
         return fwr::cuda_fail(e, "fwr_net_create");

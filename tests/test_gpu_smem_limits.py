@@ -104,3 +104,16 @@ def test_static_scratch_after_a_smaller_plan(fwr, shape):
     other.set_ctas(2)
     other.reconstruct(small, 1)
     assert torch.equal(plan.reconstruct_static(s, 1, ctas=2), ref)
+
+
+@pytest.mark.parametrize("conv", ["NET_CONV_AUTO", "NET_CONV_SIMT"])
+def test_network_after_a_narrower_one(fwr, conv):
+    plan, net, s, e = net_problem(fwr, 32, 2)
+    net.set_conv(getattr(fwr, conv))
+    ref = net.forward(plan, s).clone()
+    loss, g = net.gradients(plan, s, e)
+    fwr.Net(16, 2).close()
+    fwr.Net(4, 2).close()
+    assert torch.equal(net.forward(plan, s), ref)
+    loss2, g2 = net.gradients(plan, s, e)
+    assert loss == loss2 and np.array_equal(g, g2)
