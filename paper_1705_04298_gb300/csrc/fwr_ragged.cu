@@ -80,9 +80,9 @@ size_t ragged_smem_bytes(int N, int n) {
 }
 
 cudaError_t ragged_prepare(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(ragged_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = raise_smem_limit(ragged_kernel<1>, smem);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(ragged_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    return raise_smem_limit(ragged_kernel<2>, smem);
 }
 
 cudaError_t launch_ragged(const RaggedParams& p, int grid, size_t smem, cudaStream_t s) {

@@ -117,3 +117,24 @@ def test_network_after_a_narrower_one(fwr, conv):
     assert torch.equal(net.forward(plan, s), ref)
     loss2, g2 = net.gradients(plan, s, e)
     assert loss == loss2 and np.array_equal(g, g2)
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+def test_batch_after_a_smaller_one(fwr, shape):
+    def batch(n):
+        s, mask = slopes(n, 2, n)
+        plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=256)
+        out = torch.empty((2, 256, 256), device="cuda")
+        b = fwr.Batch([plan], [0, 0], 1)
+        b.set_shape(shape)
+        return b, s, out, fwr.Batch.pointer_table(list(s)), fwr.Batch.pointer_table(list(out))
+
+    b, s, out, sp, pp = batch(200)
+    b.run(sp, pp)
+    torch.cuda.synchronize()
+    ref = out.clone()
+    batch(60)
+    out.zero_()
+    b.run(sp, pp)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
