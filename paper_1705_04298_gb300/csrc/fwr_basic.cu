@@ -316,7 +316,7 @@ static cudaError_t launch_one(const Params<T>& p, cudaStream_t s) {
     constexpr int NT = Split<N>::NT;
     const size_t smem = smem_layout_bytes<T, N>(p.n) + (GEMM ? gemm_extra_bytes<N>() : 0);
     auto kern = basic_kernel<T, N, GEMM>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = raise_smem_limit(kern, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

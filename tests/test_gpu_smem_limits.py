@@ -138,3 +138,22 @@ def test_batch_after_a_smaller_one(fwr, shape):
     b.run(sp, pp)
     torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+def test_generic_kernel_of_several_pupils_from_several_threads(fwr):
+    """128^2 pupils above 100 lenslets run the generic kernel, whose size
+    depends on the pupil."""
+    runs = []
+    for n in (126, 101, 110, 103):
+        s, mask = slopes(n, 1, n)
+        plan = fwr.Plan(mask, 1.0, fwr.LSQ, grid=128)
+        ref = plan.reconstruct(s, 0).clone()
+        runs.append((plan, s, ref, torch.empty_like(ref), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def call(plan, s, ref, out, stream):
+        plan.reconstruct(s, 0, out, stream=stream)
+        with torch.cuda.stream(stream):
+            assert torch.equal(out, ref)
+
+    at_once([lambda r=r: call(*r) for r in runs], 2000)
