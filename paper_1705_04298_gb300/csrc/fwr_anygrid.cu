@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(AG_NT, 2) anygrid_kernel(Params<T> p, AgShape 
     V* const col = Z + line;
     const V* const s0r = s0 + li * n - off;  // dereferenced only under vbits
     const V zero = mk(T(0), T(0));
+    const bool fill_first = fills_first(p.periodic, p.iters);
     __syncthreads();
 
     bool finite = true;
@@ -290,6 +291,10 @@ __global__ void __launch_bounds__(AG_NT, 2) anygrid_kernel(Params<T> p, AgShape 
             for (int r = t / N; r < N; r += a.kt) {
                 const int c = line, i = r - off, j = c - off;
                 V v = ext ? mk(ext[r * N + c], ext[N * N + r * N + c]) : zero;
+                // Eq. PC replaces the last row's y slopes (and the last column's x
+                // slopes, which the row transforms leave out): what a warm start
+                // holds there must not reach the column sums
+                if (fill_first && r == N - 1) v.y = T(0);
                 if (i >= 0 && i < n && j >= 0 && j < n && p.mask[i * n + j]) {
                     v = mk(sl[i * n + j], sl[nn + i * n + j]);
                     finite &= isfinite(v.x) && isfinite(v.y);

@@ -74,6 +74,11 @@ template <typename... A> cudaError_t raise_smem_limit(void (*kern)(A...), size_t
 // Where Eq. PC is applied (same values as FWR_PERIODIC_* in fwr.h).
 enum : int { PERIODIC_BEFORE_EACH_FFT = 0, PERIODIC_FINAL_ONLY = 1, PERIODIC_NONE = 2 };
 
+// whether Eq. PC precedes the first transform
+__host__ __device__ __forceinline__ bool fills_first(int periodic, int iters) {
+    return periodic == PERIODIC_BEFORE_EACH_FFT || (periodic == PERIODIC_FINAL_ONLY && iters == 0);
+}
+
 // Status bits written by kernels.
 enum : unsigned { STATUS_NONFINITE = 1u, STATUS_TIMEOUT = 2u, STATUS_BADINDEX = 4u };
 
