@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(16 * N / CL, 2) cluster128_kernel(Params<float
     cluster_wait();
 
     bool finite = true;
+    const bool fill_first = fills_first(mode, p.iters);
     for (int f = int(blockIdx.x) / CL; f < p.F; f += clusters) {
         const float* const sl = p.slopes + size_t(f) * 2 * nn;
         const float* const ext = p.ext_init ? p.ext_init + size_t(f) * 2 * N * N : nullptr;
@@ -207,6 +208,8 @@ __global__ void __launch_bounds__(16 * N / CL, 2) cluster128_kernel(Params<float
                         if (e0 >= 0 && (j < e0 || j > e1)) v.y = sl[nn + ii * n + (j < e0 ? e0 : e1)];
                     }
                 }
+                // replaced by Eq. PC, as in the fused kernel
+                if (fill_first && row == N - 1) v.y = 0.f;
                 if (valid & (1u << (4 * h + i))) {
                     v = make_float2(sl[ii * n + j], sl[nn + ii * n + j]);
                     finite &= isfinite(v.x) && isfinite(v.y);

@@ -190,6 +190,7 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
     cluster_wait();
 
     bool finite = true;
+    const bool fill_first = fills_first(mode, p.iters);
     for (int f = int(blockIdx.x) / CL; f < p.F; f += clusters) {
         const double* const sl = p.slopes + size_t(f) * 2 * nn;
         const double* const ext = p.ext_init ? p.ext_init + size_t(f) * 2 * N * N : nullptr;
@@ -212,6 +213,8 @@ __global__ void __launch_bounds__(C64<N>::NT) cluster64_kernel(Params<double> p,
                     if (l >= 0 && (j < l || j > r)) x[e].y = sl[nn + i0 * n + (j < l ? l : r)];
                 }
             }
+            // replaced by Eq. PC, as in the fused kernel
+            if (fill_first && row == N - 1) x[e].y = 0.0;
             if (valid[e]) {
                 meas[e] = make_double2(sl[i0 * n + j], sl[nn + i0 * n + j]);
                 finite &= isfinite(meas[e].x) && isfinite(meas[e].y);

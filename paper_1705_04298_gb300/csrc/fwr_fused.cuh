@@ -514,7 +514,10 @@ __device__ __forceinline__ bool fused_frame(const FusedCtx<T, N>& c, const T* sl
     const bool warm = ext || exth;
     if (warm) {
         // warm start: coalesced 4-wide loads of both channels, staged in Z
-        // (free between frames) as complex cells
+        // (free between frames) as complex cells. Where Eq. PC comes before the
+        // first transform it replaces the last row's y slopes (and the last
+        // column's x slopes): they must not reach the column sums it is made of
+        const bool fill_first = fills_first(mode, iters);
         for (int q = tid; q < N * N / 4; q += NT) {
             const int rr = q / (N / 4), cc = 4 * (q - rr * (N / 4));
             T ex[4], ey[4];
@@ -525,6 +528,7 @@ __device__ __forceinline__ bool fused_frame(const FusedCtx<T, N>& c, const T* sl
                 load_row4(exth + rr * N + cc, ex);
                 load_row4(exth + N * N + rr * N + cc, ey);
             }
+            if (fill_first && rr == N - 1) ey[0] = ey[1] = ey[2] = ey[3] = T(0);
             // two 16-byte stores per four cells (single cells at a 32-byte lane
             // stride would conflict eight ways)
             T* const zp = reinterpret_cast<T*>(Z + rr * S + cc);

@@ -22,9 +22,12 @@ def fwr():
     return m
 
 
-# window grids with odd and even N/2; a 128^2 pupil of the generic kernel
+# window grids with odd and even N/2; 128^2 pupils of the generic kernel, and of
+# the fused and the cluster kernel (many and few frames)
 @pytest.mark.parametrize("N,n,F,precision", [(46, 40, 2, "fp32"), (20, 14, 3, "fp32"), (46, 40, 500, "fp32"),
-                                             (26, 20, 2, "fp64"), (128, 110, 2, "fp32")])
+                                             (26, 20, 2, "fp64"), (128, 110, 2, "fp32"), (128, 91, 2, "fp32"),
+                                             (128, 91, 60, "fp32"), (128, 40, 2, "fp32"), (128, 40, 60, "fp32"),
+                                             (32, 16, 2, "fp32"), (32, 16, 2, "fp64"), (64, 31, 130, "fp64")])
 @pytest.mark.parametrize("k,periodic", [(2, 0), (0, 1)])
 @pytest.mark.parametrize("value", [float("nan"), 1e30])
 def test_fill_cells_of_a_warm_start_are_replaced(fwr, N, n, F, precision, k, periodic, value):
