@@ -547,6 +547,18 @@ static fwr_status check_call(const fwr_plan* p, const void* slopes, int n_frames
 // the warm start is read with 16-byte vector loads (NULL passes)
 static bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; }
 
+// Whether an FP32 FFT call on N <= 128 takes the fused kernel (and the cluster
+// kernel, whose bits are the same) rather than the generic one. Pupils of 83 to
+// 100 lenslets on 128^2 do where its rounding error is the smaller one: Eq. PC
+// before every transform and two iterations or more, 0.74 to 0.98 of the
+// generic kernel's over n, warm starts and ext_out. With fewer iterations (1.01
+// to 1.10) and the other placements of Eq. PC (0.85 to 1.17, the extended
+// slopes up to 1.33) the generic kernel, half as fast, is the more accurate.
+static bool takes_fused(const fwr_plan* p, int iters) {
+    if (!fwr::fused_fits(p->N, 4, p->n)) return false;
+    return fwr::fused_supported(p->N, 4, p->n) || (p->periodic == FWR_PERIODIC_BEFORE_EACH_FFT && iters >= 2);
+}
+
 fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext_init, int n_frames, int iters,
                               float* phase, float* ext_out, void* stream) {
     fwr_status st = check_call(p, slopes, n_frames, iters, phase, ext_out);
@@ -590,14 +602,14 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     } else if (p->N >= 256) {
         if (ext_out || !phase) return FWR_ERR_UNSUPPORTED;
         e = fwr::launch_slab(p->N, k, p->d_scratch, p->d_counters, p->scratch_ctas, static_cast<cudaStream_t>(stream));
-    } else if (p->N == 128 && phase && !ext_out && p->ctas == 0 && fwr::fused_fits(128, 4, p->n) &&
+    } else if (p->N == 128 && phase && !ext_out && p->ctas == 0 && takes_fused(p, iters) &&
                fwr::cluster128_wanted(n_frames, p->sms)) {
         // few frames on every SM (no FWR_OPT_CTAS); pupils that the fused kernel
         // takes, whose bits these are
         e = fwr::launch_cluster_f32(k, p->sms, static_cast<cudaStream_t>(stream));
     } else {
-        e = fwr::fused_fits(p->N, 4, p->n) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
-                                           : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
+        e = takes_fused(p, iters) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
+                                  : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
     }
     return e == cudaSuccess ? FWR_OK : cuda_fail(e, "gerchberg launch");
 }
