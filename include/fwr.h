@@ -162,7 +162,9 @@ typedef enum {
  *     frame (128x128: a cluster of CTAs; 256x256 and 512x512: a cooperative
  *     launch, whose CTAs must all be resident); any other value keeps one CTA
  *     per frame. (The FP64 entry point does the same on 32x32 and 64x64, where
- *     the two agree to rounding.)
+ *     the two agree to rounding.) A value or shape chosen by fwr_plan_autotune
+ *     holds for calls of at least the frames it was tuned with; calls of fewer
+ *     frames keep the paths for few frames.
  */
 #define FWR_OPT_SHAPE 6
 #define FWR_OPT_CTAS 7

@@ -480,6 +480,7 @@ fwr_status fwr_plan_set_option(fwr_plan* p, int key, double value) {
         const int v = int(value);
         if (double(v) != value || v < 0 || v > 2) return FWR_ERR_ARG;
         p->shape = v;
+        p->tuned_frames = 0;
         return FWR_OK;
     }
     if (key == FWR_OPT_L2_PERSIST) {
@@ -523,6 +524,7 @@ fwr_status fwr_plan_set_option(fwr_plan* p, int key, double value) {
         const int v = int(value);
         if (double(v) != value || v < 0 || v > 65536) return FWR_ERR_ARG;
         p->ctas = v;
+        p->tuned_frames = 0;
         return FWR_OK;
     }
     if (key == FWR_OPT_PERIODIC) {
@@ -579,6 +581,7 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     k.periodic = p->periodic;
     k.shape = p->shape;
     k.ctas = p->ctas;
+    k.one_cta = (p->one_cta(n_frames) || (p->shape == 1 && n_frames >= p->tuned_frames)) ? 1 : 0;
     k.l2_bytes = p->l2_bytes;
     k.l2_hit = p->l2_hit;
     k.status = p->d_status;
@@ -602,10 +605,10 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     } else if (p->N >= 256) {
         if (ext_out || !phase) return FWR_ERR_UNSUPPORTED;
         e = fwr::launch_slab(p->N, k, p->d_scratch, p->d_counters, p->scratch_ctas, static_cast<cudaStream_t>(stream));
-    } else if (p->N == 128 && phase && !ext_out && p->ctas == 0 && takes_fused(p, iters) &&
+    } else if (p->N == 128 && phase && !ext_out && !p->one_cta(n_frames) && takes_fused(p, iters) &&
                fwr::cluster128_wanted(n_frames, p->sms)) {
-        // few frames on every SM (no FWR_OPT_CTAS); pupils that the fused kernel
-        // takes, whose bits these are
+        // few frames on every SM (no FWR_OPT_CTAS of the caller's); pupils that
+        // the fused kernel takes, whose bits these are
         e = fwr::launch_cluster_f32(k, p->sms, static_cast<cudaStream_t>(stream));
     } else {
         e = takes_fused(p, iters) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
@@ -699,8 +702,8 @@ fwr_status fwr_reconstruct_f64(fwr_plan* p, const double* slopes, const double* 
         k.hud = p->d_hud;
     }
     cudaError_t e = !pow2(p->N) ? fwr::launch_anygrid_f64(p->N, k, static_cast<cudaStream_t>(stream))
-                    // few frames on every SM (no FWR_OPT_CTAS)
-                    : phase && !ext_out && p->ctas == 0 && fwr::cluster64_wanted(p->N, n_frames, p->sms)
+                    // few frames on every SM (no FWR_OPT_CTAS of the caller's)
+                    : phase && !ext_out && !p->one_cta(n_frames) && fwr::cluster64_wanted(p->N, n_frames, p->sms)
                         ? fwr::launch_cluster_f64(p->N, k, static_cast<cudaStream_t>(stream))
                     : fwr::fused_supported(p->N, 8, p->n)
                         ? fwr::launch_fused_f64(p->N, k, static_cast<cudaStream_t>(stream))
@@ -890,7 +893,7 @@ cudaError_t fwr::launch_warm_bf16(fwr_plan* p, const float* slopes, const uint16
     k.shape = p->shape;
     k.ctas = p->ctas;
     k.status = p->d_status;
-    if (p->N == 128 && p->ctas == 0 && fwr::cluster128_wanted(n_frames, p->sms))
+    if (p->N == 128 && !p->one_cta(n_frames) && fwr::cluster128_wanted(n_frames, p->sms))
         return fwr::launch_cluster_f32(k, p->sms, s);
     k.pdl = pdl ? 1 : 0;
     return fwr::launch_fused_f32(p->N, k, s);

@@ -57,6 +57,11 @@ struct fwr_plan {
     size_t l2_bytes = 0;            // its access-policy window over d_scratch
     float l2_hit = 0.f;
     int ctas = 0;                   // persistent CTAs (FWR_OPT_CTAS; 0 = every SM)
+    // frames per call that fwr_plan_autotune chose shape and ctas for (0: the
+    // caller set them): calls of fewer frames keep the paths for few frames
+    int tuned_frames = 0;
+    // whether a call keeps to one CTA per frame
+    bool one_cta(int n_frames) const { return ctas != 0 && n_frames >= tuned_frames; }
     int16_t* d_hud = nullptr;       // [4][n]: pupil edges per column and row (Hudgin extension)
     double pixel = 0.0;             // d_px / d of the filter tables
     int device = 0;

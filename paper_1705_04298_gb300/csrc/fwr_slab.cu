@@ -149,7 +149,7 @@ cudaError_t launch_team(int N, int team, const Params<float>& p, float2* scratch
 cudaError_t launch_slab(int N, const Params<float>& p, float2* scratch, unsigned* counters, int max_ctas,
                         cudaStream_t s) {
     if (N != 256 && N != 512) return cudaErrorInvalidValue;
-    if (p.ctas == 0 && p.l2_bytes == 0 && p.shape != 1) {
+    if (!p.one_cta && p.l2_bytes == 0) {
         const int team = team_size(N, p.F, max_ctas);
         if (team > 1) {
             cudaError_t e = launch_team(N, team, p, scratch, counters, max_ctas, s);

@@ -27,8 +27,11 @@ std::string tune_key(const fwr_plan* p, int n_frames, int iters) {
     cudaDriverGetVersion(&drv);
     cudaRuntimeGetVersion(&rt);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    // kern: raised with every change of the kernels that can change the choice
+    // (2: few frames share a frame between SMs), so that an earlier library's
+    // entries are timed again
     std::ostringstream k;
-    k << prop.name << "|sm" << sms << "|drv" << drv << "|rt" << rt << "|N" << p->N << "n" << p->n << "v"
+    k << "kern2|" << prop.name << "|sm" << sms << "|drv" << drv << "|rt" << rt << "|N" << p->N << "n" << p->n << "v"
       << p->nvalid << "|t" << p->transform << "p" << p->periodic << "f" << p->filter << "e" << p->extension << "g"
       << p->g_model << "x" << p->pixel << "|F" << n_frames << "|k" << iters;
     std::string s = k.str();
@@ -92,6 +95,7 @@ fwr_status fwr_plan_autotune(fwr_plan* p, const float* slopes, int n_frames, int
     if (cached(cache_path, key, &shape, &ctas, &persist)) {
         p->shape = shape;
         p->ctas = ctas;
+        p->tuned_frames = n_frames;
         fwr_status st = FWR_OK;
         if (persist != p->l2_persist) st = fwr_plan_set_option(p, FWR_OPT_L2_PERSIST, persist);
         cudaSetDevice(prev);
@@ -111,10 +115,11 @@ fwr_status fwr_plan_autotune(fwr_plan* p, const float* slopes, int n_frames, int
     // timing the plan alone cannot weigh
     std::vector<int> persist_opts = {p->l2_persist};
     std::vector<int> ctas_opts = {0};
-    if (sms >= 8) {
-        ctas_opts.push_back(3 * sms / 4);
-        ctas_opts.push_back(sms / 2);
-    }
+    // caps that these frames reach: a larger one is the same launch, and chosen
+    // by the noise of the timing it would hold for other calls of the plan
+    if (sms >= 8)
+        for (int c : {3 * sms / 4, sms / 2})
+            if (c < n_frames) ctas_opts.push_back(c);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e;
@@ -123,7 +128,8 @@ fwr_status fwr_plan_autotune(fwr_plan* p, const float* slopes, int n_frames, int
         cudaSetDevice(prev);
         return fwr::cuda_fail(e, "fwr_plan_autotune events");
     }
-    const int old_shape = p->shape, old_ctas = p->ctas, old_persist = p->l2_persist;
+    const int old_shape = p->shape, old_ctas = p->ctas, old_persist = p->l2_persist, old_tuned = p->tuned_frames;
+    p->tuned_frames = 0;  // each candidate is taken at its word
     double best = 1e30;
     int best_shape = old_shape, best_ctas = old_ctas, best_persist = old_persist;
     fwr_status st = FWR_OK;
@@ -168,12 +174,14 @@ fwr_status fwr_plan_autotune(fwr_plan* p, const float* slopes, int n_frames, int
     if (st != FWR_OK) {
         p->shape = old_shape;
         p->ctas = old_ctas;
+        p->tuned_frames = old_tuned;
         fwr_plan_set_option(p, FWR_OPT_L2_PERSIST, old_persist);
         cudaSetDevice(prev);
         return st;
     }
     p->shape = best_shape;
     p->ctas = best_ctas;
+    p->tuned_frames = n_frames;
     if (best_persist != p->l2_persist) fwr_plan_set_option(p, FWR_OPT_L2_PERSIST, best_persist);
     if (cache_path && cache_path[0]) {
         std::ofstream o(cache_path, std::ios::app);
