@@ -185,6 +185,18 @@ typedef enum {
  * same either way. Opt-in only: fwr_plan_autotune keeps the caller's setting.
  */
 #define FWR_OPT_L2_PERSIST 8
+/*
+ * FWR_OPT_TEAM_WAIT (256x256 and 512x512 plans; FWR_ERR_UNSUPPORTED for
+ * others): how long, in GPU clock cycles, the CTAs that share a frame of a call
+ * of few frames (FWR_OPT_CTAS) wait for one another at most; default 4e9, about
+ * two seconds; 0 to 1e15. They are all resident, so the bound is only reached
+ * when the GPU is taken from the process for that long. The call's phases are
+ * then unfinished and the status word says FWR_ERR_TIMEOUT; until
+ * fwr_get_status has read it, further calls of few frames on the plan write no
+ * phase (fwr_reconstruct_host copies out what its staging memory held), though
+ * they return FWR_OK.
+ */
+#define FWR_OPT_TEAM_WAIT 9
 
 /*
  * Create a plan for an n x n lenslet array (Sec. 2; Algorithm 1 input).
@@ -537,8 +549,10 @@ fwr_status fwr_dft2_bf16x3(int N, const float* in_dev, float* out_dev, int n_fra
 
 /*
  * Read and clear the plan's sticky device status word. Synchronises the
- * plan's device. FWR_OK, FWR_ERR_NONFINITE, FWR_ERR_TIMEOUT or (ragged
- * launches given an invalid plan index) FWR_ERR_ARG.
+ * plan's device. FWR_OK, FWR_ERR_TIMEOUT (FWR_OPT_TEAM_WAIT: phases not
+ * written, calls of few frames suspended until now), FWR_ERR_NONFINITE or
+ * (ragged launches given an invalid plan index) FWR_ERR_ARG, in this order if
+ * several are set.
  */
 fwr_status fwr_get_status(fwr_plan* plan);
 

@@ -527,6 +527,12 @@ fwr_status fwr_plan_set_option(fwr_plan* p, int key, double value) {
         p->tuned_frames = 0;
         return FWR_OK;
     }
+    if (key == FWR_OPT_TEAM_WAIT) {
+        if (!(value >= 0.0 && value <= 1e15)) return FWR_ERR_ARG;
+        if (!p->d_counters) return FWR_ERR_UNSUPPORTED;
+        p->team_wait = static_cast<long long>(value);
+        return FWR_OK;
+    }
     if (key == FWR_OPT_PERIODIC) {
         const int v = int(value);
         if (double(v) != value || v < FWR_PERIODIC_BEFORE_EACH_FFT || v > FWR_PERIODIC_NONE) return FWR_ERR_ARG;
@@ -582,6 +588,7 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     k.shape = p->shape;
     k.ctas = p->ctas;
     k.one_cta = (p->one_cta(n_frames) || (p->shape == 1 && n_frames >= p->tuned_frames)) ? 1 : 0;
+    k.team_wait = p->team_wait;
     k.l2_bytes = p->l2_bytes;
     k.l2_hit = p->l2_hit;
     k.status = p->d_status;
@@ -853,8 +860,9 @@ fwr_status fwr_get_status(fwr_plan* p) {
     if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(unsigned));
     cudaSetDevice(prev);
     if (e != cudaSuccess) return cuda_fail(e, "status read");
-    if (v & fwr::STATUS_NONFINITE) return FWR_ERR_NONFINITE;
+    // a wait that ran out left phases unwritten: it goes first
     if (v & fwr::STATUS_TIMEOUT) return FWR_ERR_TIMEOUT;
+    if (v & fwr::STATUS_NONFINITE) return FWR_ERR_NONFINITE;
     if (v & fwr::STATUS_BADINDEX) return FWR_ERR_ARG;
     return FWR_OK;
 }

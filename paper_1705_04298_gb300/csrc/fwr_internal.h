@@ -45,6 +45,7 @@ template <typename T> struct Params {
     // read from L2 (0: 1)
     int shape = 0;
     int ctas = 0;   // persistent CTAs (0: every SM, times the resident CTAs per SM)
+    long long team_wait = 0;  // slab kernel, a team of CTAs per frame: bound of a barrier's wait (clock cycles)
     int one_cta = 0;  // slab kernel: one CTA per frame, however few the frames
     // slab kernel: an L2 access-policy window over the scratch (FWR_OPT_L2_PERSIST),
     // persisting hits for l2_hit of its l2_bytes; l2_bytes = 0: none

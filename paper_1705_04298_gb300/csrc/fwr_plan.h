@@ -60,6 +60,7 @@ struct fwr_plan {
     // frames per call that fwr_plan_autotune chose shape and ctas for (0: the
     // caller set them): calls of fewer frames keep the paths for few frames
     int tuned_frames = 0;
+    long long team_wait = 4000000000ll;  // FWR_OPT_TEAM_WAIT
     // whether a call keeps to one CTA per frame
     bool one_cta(int n_frames) const { return ctas != 0 && n_frames >= tuned_frames; }
     int16_t* d_hud = nullptr;       // [4][n]: pupil edges per column and row (Hudgin extension)

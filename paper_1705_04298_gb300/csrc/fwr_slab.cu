@@ -49,7 +49,7 @@ slab_team_kernel(Params<float> p, float2* scratch, unsigned* counters, int team)
     slab_setup<N>(c, smem, p.tab, p.mask, p.n, p.off, p.periodic);
     const int teams = int(gridDim.x) / team, id = int(blockIdx.x) % teams, rank = int(blockIdx.x) / teams;
     float2* G = scratch + size_t(id) * N * N;
-    TeamBar bar{counters + id * TEAM_COUNTER_STRIDE, 0u, team, false};
+    TeamBar bar{counters + id * TEAM_COUNTER_STRIDE, 0u, team, p.team_wait, false};
     const int nn = p.n * p.n;
     bool finite = true;
     for (int f = id; f < p.F && !bar.dead; f += teams)

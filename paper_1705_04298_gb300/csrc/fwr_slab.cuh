@@ -122,15 +122,15 @@ __device__ __forceinline__ void group_sync(int g, int threads) {
 
 // Barrier of the CTAs that share a frame (all resident: a cooperative launch):
 // `count` is a counter in global memory that each CTA raises once per barrier,
-// and that team_leave returns to zero. The wait is bounded: after about two
-// seconds the CTA gives up and every thread gets false.
+// and that team_leave returns to zero. The wait is bounded: after `wait`
+// clock cycles (FWR_OPT_TEAM_WAIT) the CTA gives up and every thread gets false.
 struct TeamBar {
     unsigned* count;   // [0]: arrivals, [1]: CTAs done (nullptr: no team)
     unsigned target;   // arrivals that complete the next barrier
     int team;
+    long long wait;
     bool dead;         // a wait ran out
 };
-constexpr long long TEAM_WAIT = 4000000000ll;  // clock cycles
 
 __device__ __forceinline__ bool team_sync(TeamBar& b) {
     __syncthreads();
@@ -144,7 +144,7 @@ __device__ __forceinline__ bool team_sync(TeamBar& b) {
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(b.count) : "memory");
             ok = v >= b.target;
-        } while (!ok && clock64() - t0 < TEAM_WAIT);
+        } while (!ok && clock64() - t0 < b.wait);
         __threadfence();
     }
     b.dead = !__syncthreads_and(ok);

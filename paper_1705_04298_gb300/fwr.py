@@ -30,6 +30,7 @@ OPT_EXTENSION = 5
 OPT_SHAPE = 6
 OPT_CTAS = 7
 OPT_L2_PERSIST = 8
+OPT_TEAM_WAIT = 9
 EXT_ZERO = 0
 EXT_HUDGIN = 1
 TRANSFORM_FFT = 0
@@ -227,6 +228,11 @@ class Plan:
     def set_ctas(self, ctas):
         """Persistent CTAs of a launch (FWR_OPT_CTAS; 0 = every SM)."""
         _check(self._lib.fwr_plan_set_option(self._h, OPT_CTAS, float(ctas)), "fwr_plan_set_option")
+
+    def set_team_wait(self, cycles):
+        """Bound, in GPU clock cycles, of the waits between the CTAs that share a
+        frame of a 256^2 / 512^2 plan (FWR_OPT_TEAM_WAIT)."""
+        _check(self._lib.fwr_plan_set_option(self._h, OPT_TEAM_WAIT, float(cycles)), "fwr_plan_set_option")
 
     @property
     def shape(self):
