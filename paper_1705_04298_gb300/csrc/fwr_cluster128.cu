@@ -377,8 +377,13 @@ __global__ void __launch_bounds__(16 * N / CL, 2) cluster128_kernel(Params<float
 // Frames that run at once: 7 with clusters of 16 CTAs, 30 with 8 (two CTAs per
 // SM); the fused kernel takes a frame per SM in the time of one. Measured, k = 5
 // (us, clusters of 16 / of 8 / fused kernel): 1 to 7 frames 28 / 37 / 68, 15: 62 /
-// 39 / 68, 30: 94 / 57 / 68, 40: - / 89 / 68.
-bool cluster128_wanted(int F, int sms) { return F <= sms / 5; }
+// 39 / 68, 30: 94 / 57 / 68, 40: - / 89 / 68. A call cannot know what other
+// streams run, and a cluster takes more SM time per frame (2.6 to 4 us of the
+// chip against 0.5): several calls at once, in sum (us, this / fused kernel; a
+// graph with parallel branches): 10 x 1 frames 48 / 82, 64 x 1 217 / 225, 5 x 4
+// 65 / 74, 10 x 4 111 / 83, 2 x 15 56 / 70, 5 x 15 142 / 74, 2 x 30 111 / 70, 5 x
+// 30 257 / 74. So the line lies at 15 frames, where a lone call gains 1.7 times.
+bool cluster128_wanted(int F, int sms) { return F <= sms / 10; }
 
 template <int CL> static cudaError_t launch_cl(const Params<float>& p, cudaStream_t s) {
     static std::mutex mu;
