@@ -91,13 +91,6 @@ __device__ __forceinline__ void load2(const double2* p, double2& a, double2& b) 
     b = p[1];
 }
 
-template <typename V> __device__ __forceinline__ V cmul_w(V a, V b) {
-    return mk(fmadd(a.x, b.x, -mulrn(a.y, b.y)), fmadd(a.x, b.y, mulrn(a.y, b.x)));
-}
-template <typename V> __device__ __forceinline__ V cmulc_w(V a, V b) {  // conj(a) b
-    return mk(fmadd(a.x, b.x, mulrn(a.y, b.y)), fmadd(a.x, b.y, -mulrn(a.y, b.x)));
-}
-
 // The sums of one line for k = k0 .. k0 + K - 1: P = sum a_j cos, Q = sum b_j
 // sin of the even (e) and odd (o) elements.
 template <typename V, int K> struct AgSums {
@@ -173,14 +166,14 @@ __device__ __forceinline__ void ag_outputs(const AgSums<V, K>& s, const AgShape&
         const V om = mk(po.x + qo.y, po.y - qo.x), op = mk(po.x - qo.y, po.y + qo.x);
         const V e1 = INV ? ep : em, e2 = INV ? em : ep, o1 = INV ? op : om, o2 = INV ? om : op;
         const V w1 = tw[k];
-        V t = INV ? cmulc_w(w1, o1) : cmul_w(o1, w1);
-        if (FILL) t = cadd(t, cmulc_w(w1, d));
+        V t = INV ? cmulc_rn(w1, o1) : cmul_rn(o1, w1);
+        if (FILL) t = cadd(t, cmulc_rn(w1, d));
         f(k, cadd(e1, t), 4 * i);
         f(k + a.M, csub(e1, t), 4 * i + 1);
         if (k != 0 && 2 * k != a.M) {
             const V w2 = tw[a.M - k];
-            t = INV ? cmulc_w(w2, o2) : cmul_w(o2, w2);
-            if (FILL) t = cadd(t, cmulc_w(w2, d));
+            t = INV ? cmulc_rn(w2, o2) : cmul_rn(o2, w2);
+            if (FILL) t = cadd(t, cmulc_rn(w2, d));
             f(a.M - k, cadd(e2, t), 4 * i + 2);
             f(a.N - k, csub(e2, t), 4 * i + 3);
         }
@@ -194,14 +187,9 @@ __device__ __forceinline__ void ag_final(V* Z, const Tables<T>& tab, const uint3
     for (int p = t; p < a.NP; p += a.tpf) {
         const int a1 = pa[p] & 0xFFFF, a2 = pa[p] >> 16, ky = a1 / a.S, kx = a1 - ky * a.S;
         const V z1 = Z[a1], z2 = Z[a2];
-        const V sx = mk(half * (z1.x + z2.x), half * (z1.y - z2.y));
-        const V sy = mk(half * (z1.y + z2.y), half * (z2.x - z1.x));
-        const V gx = cmul(tab.A[kx], tab.Tt[ky]);
-        const V gy = cmul(tab.Tt[kx], tab.A[ky]);
-        const T w = tab.wfin[ky * a.N + kx];
-        const V ph = cadd(cmulc(gx, sx), cmulc(gy, sy));
-        Z[a2] = mk(ph.x * w, -ph.y * w);
-        Z[a1] = mk(ph.x * w, ph.y * w);
+        const V ph = final_bin(z1, z2, tab.A[kx], tab.Tt[kx], tab.A[ky], tab.Tt[ky], half * tab.wfin[ky * a.N + kx]);
+        Z[a2] = mk(ph.x, -ph.y);
+        Z[a1] = ph;
     }
 }
 
@@ -252,9 +240,10 @@ __global__ void __launch_bounds__(AG_NT, 2) anygrid_kernel(Params<T> p, AgShape 
         pa[q] = uint32_t(ky * S + kx) | uint32_t(my * S + mx) << 16;
         const T w = p.tab.iota[ky * N + kx];
         const T *u = p.tab.pt + 4 * kx, *v = p.tab.pt + 4 * ky, *un = p.tab.pt + 4 * mx, *vn = p.tab.pt + 4 * my;
-        T al, be, ga, al2, be2, ga2;
+        T al, be, ga, al2, none;
         lsq_coefs(w, u[0], u[1], T(0.5) * u[2], T(0.5) * u[3], quad<T>{v[0], v[1], v[2], v[3]}, al, be, ga);
-        lsq_coefs(w, un[0], un[1], T(0.5) * un[2], T(0.5) * un[3], quad<T>{vn[0], vn[1], vn[2], vn[3]}, al2, be2, ga2);
+        lsq_coefs(w, un[0], un[1], T(0.5) * un[2], T(0.5) * un[3], quad<T>{vn[0], vn[1], vn[2], vn[3]}, al2, none,
+                  none);
         cf[q] = Quad<T>{al, be, ga, al2};
     }
     // roles: line, first k
