@@ -465,8 +465,9 @@ void fwr_ragged_release(void);
  *                    BF16; they differ only in summation order. The same holds
  *                    for the backward pass, whose FP32 gradients enter the
  *                    tensor cores as three exact BF16 parts (layers with input
- *                    and output channels multiples of 16). Unknown option or
- *                    value: FWR_ERR_ARG.
+ *                    and output channels multiples of 16; the weight gradient
+ *                    of the first layer too, its three input channels padded).
+ *                    Unknown option or value: FWR_ERR_ARG.
  * fwr_net_tc_layers  how many layers are eligible for the tensor-core forward
  *                    (-1 for NULL).
  */

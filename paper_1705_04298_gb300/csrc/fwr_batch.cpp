@@ -102,7 +102,7 @@ fwr_status fwr_batch_create(fwr_batch** out, fwr_plan* const* plans, int n_plans
         const size_t b = fwr::ragged_smem_bytes(p->N, p->n);
         if (b == 0 || b > size_t(227) * 1024) {
             fwr::set_last_error("fwr_batch_create: ragged batches take 128x128 and 256x256 plans "
-                                "(128x128 with at most 85 lenslets across)");
+                                "(128x128 with at most 82 lenslets across)");
             return FWR_ERR_UNSUPPORTED;
         }
         smem = std::max(smem, b);

@@ -321,7 +321,9 @@ template <int N> cudaError_t launch_n(const Params<double>& p, cudaStream_t s) {
 // Up to 15 frames run at once, more take turns, while the fused kernel takes a
 // frame per SM in the time of one. Measured at k = 10 (us, this / fused): 32^2,
 // 76 frames: 204 / 326, 100: 261 / 326, 152: 360 / 327; 64^2, 76 frames: 835 / 1098,
-// 100: 1019 / 1097.
+// 100: 1019 / 1097. Several such calls at once cost more SM time than one CTA per
+// frame: 38 frames on 32^2 alone 131 / 324, two at once 202 / 325, four 383 / 326,
+// eight 716 / 498; single frames gain on any number of streams (64: 272 / 987).
 bool cluster64_wanted(int N, int F, int sms) {
     return N == 32 ? F <= 3 * sms / 4 : N == 64 ? F <= 2 * sms / 3 : false;
 }

@@ -152,7 +152,8 @@ cudaError_t launch_anygrid_f64(int N, const Params<double>& p, cudaStream_t s);
 // Main fused kernel (fwr_fused.cu). fused_supported() says whether all of its
 // tables fit shared memory on grid N with n lenslets for the element size (what
 // the Hudgin extension, warm starts in BF16 and ragged batches ask for);
-// fused_fits() whether it runs: FP32 on 128^2 keeps one table in tensor memory
+// fused_fits() whether it can run (fwr_api.cpp's takes_fused() says when it
+// does): FP32 on 128^2 keeps one table in tensor memory
 // instead, so 83 to 100 lenslets across run too (1000 frames of 100 x 100, k =
 // 10: 1715 us by the basic kernel, 813 here; one frame 242 and 46).
 bool fused_supported(int N, int elem_bytes, int n);

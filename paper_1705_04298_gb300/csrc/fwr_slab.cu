@@ -95,18 +95,18 @@ namespace {
 // on 256^2 and 200 x 200 on 512^2 lenslets, five iterations, 152 SMs; 1 is
 // slab_kernel; 8 and 32 slabs, two per CTA and step): a wave takes the same
 // time with fewer frames, so the least number of waves times their cost wins.
-// (512^2: all taken on one earlier version of the kernel; 1, 6, 8 and 16 have
-// fallen by 6 to 10 % since.)
 // At 512^2 teams of 8 also win for many frames: 19 grids of 2 MB in flight stay
 // in L2, 152 do not. Measured with / without teams: 256^2, F = 1: 142 / 398,
 // F = 38: 157 / 398, F = 200: 753 / 855; 512^2, F = 1: 181 / 2043, F = 16: 312 /
-// 2047, F = 76: 1238 / 2470, F = 152: 2475 / 2741.
+// 2047, F = 76: 1238 / 2470, F = 152: 2475 / 2741. Several calls at once: 256^2,
+// 8 of F = 1: 157 / 406, 2 of F = 38: 314 / 402, 4 of F = 38: 631 / 461; 512^2, 8 of
+// F = 16: 2559 / 2647.
 int team_size(int N, int F, int ctas) {
     struct Cost {
         int team, us;
     };
-    static const Cost c256[] = {{1, 458}, {2, 257}, {4, 157}};
-    static const Cost c512[] = {{1, 2911}, {2, 1473}, {3, 990}, {4, 708}, {6, 485}, {8, 341}, {16, 197}};
+    static const Cost c256[] = {{1, 460}, {2, 259}, {4, 160}};
+    static const Cost c512[] = {{1, 2749}, {2, 1370}, {3, 937}, {4, 638}, {6, 443}, {8, 316}, {16, 186}};
     const Cost* c = N == 512 ? c512 : c256;
     const int nc = N == 512 ? 7 : 3;
     int best = 1;
