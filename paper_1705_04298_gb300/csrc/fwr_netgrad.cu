@@ -103,12 +103,15 @@ WgradShape wgrad_shape(int cin, int cout, int H) {
     return w;
 }
 
-// chunks of image rows (one CTA each): two CTAs per SM, at least one stage of rows each
+// chunks of image rows (one CTA each): two CTAs per SM, whole turns of the
+// copies where there is more than one. (A few images do not fill the copies of
+// one CTA; they are spread all the same: one image of width 3, 12 x 32 x 32, 29
+// us in one CTA, 7 in 32.)
 int wgrad_rows(const WgradShape& w, long long rows, int sms) {
     const long long want = std::max(1, 2 * sms / w.ny);
     long long r = (rows + want - 1) / want;
     const int unit = w.S < w.RS ? w.S : w.RS;
-    r = (r + unit - 1) / unit * unit;
+    if (r > unit) r = (r + unit - 1) / unit * unit;
     return int(r);
 }
 
@@ -233,11 +236,11 @@ k_wgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ A, int
             }
         }
     }
-    // sum the S copies, pairwise halves, one kernel column at a time
-    const int tl = tid % w.TG;
+    // sum the copies (those that had a row), pairwise halves, one kernel column at a time
+    const int tl = tid % w.TG, copies = min(w.S, rows_cta);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        for (int n = w.S; n > 1; n = (n + 1) / 2) {
+        for (int n = copies; n > 1; n = (n + 1) / 2) {
             const int half = (n + 1) / 2;
             u64* const red = reinterpret_cast<u64*>(sm);  // [copy][tile][21]
             __syncthreads();
@@ -343,6 +346,7 @@ constexpr size_t DGRAD_SMEM = 100 * 1024;
 
 struct DgradShape {
     int cb, ny, pairs, S, threads, slots, portion;  // portion: row pairs per image part
+    int block;  // threads of the launch: those beyond `threads` stage only
     size_t smem;
 };
 
@@ -376,6 +380,8 @@ DgradShape dgrad_shape(int cin, int H, long long total_pairs, int sms) {
     d.portion = d.pairs < img ? d.pairs : img;
     d.slots = slots(d.pairs);
     d.threads = d.cb * per_pair * d.pairs * d.S;
+    // CTAs that have an SM each get a few more warps for the staging
+    d.block = (total_pairs + d.pairs - 1) / d.pairs * d.ny <= sms ? std::max(d.threads, 128) : d.threads;
     d.smem = std::max(bytes(d.pairs), size_t(d.threads / 2) * 33 * sizeof(u64));
     return d;
 }
@@ -391,7 +397,7 @@ k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, in
     float* const zs = sm;                                     // [slots][DG_CO][ZS], column x at 4 + x
     float* const wsm = sm + size_t(d.slots) * DG_CO * ZS;     // [DG_CO][9][n8]
     constexpr int img = H / 2;
-    const int tid = threadIdx.x, tt = blockDim.x / d.S, sp = tid / tt, tl = tid - sp * tt;
+    const int tid = threadIdx.x, tt = d.threads / d.S, sp = tid / tt, tl = tid - sp * tt;
     const int cib = tl % d.cb, tile = tl / d.cb;
     const int xt = tile % (W / 4), pr = tile / (W / 4);       // tile column, row pair in the CTA
     const int pair0 = blockIdx.x * d.pairs, ci0 = blockIdx.y * n8;
@@ -431,17 +437,26 @@ k_dgrad3(const float* __restrict__ dZ, int cout, const bf16* __restrict__ Wt, in
             o[2 * ZS] = v.z;
             o[3 * ZS] = v.w;
         }
-        // weight rows (output channel, tap): two rows per warp at a time, 16 lanes each
-        for (int ct = tid >> 4; ct < nc * 9; ct += blockDim.x >> 4) {
-            const bf16* src = Wt + (size_t(c0) * 9 + ct) * cin + ci0;
+        // weight rows (output channel, tap): two rows per warp at a time, 16 lanes
+        // each; several loads in flight, along the row where it is long, over the
+        // rows where it is short
+        const bf16* const wsrc = Wt + size_t(c0) * 9 * cin + ci0;
+        if (n8 > 32) {
+            for (int ct = tid >> 4; ct < nc * 9; ct += blockDim.x >> 4)
 #pragma unroll 4
-            for (int c = tid & 15; c < n8; c += 16) wsm[ct * n8 + c] = ci0 + c < cin ? __bfloat162float(src[c]) : 0.f;
+                for (int c = tid & 15; c < n8; c += 16)
+                    wsm[ct * n8 + c] = ci0 + c < cin ? __bfloat162float(wsrc[size_t(ct) * cin + c]) : 0.f;
+        } else {
+            for (int c = tid & 15; c < n8; c += 16)
+#pragma unroll 8
+                for (int ct = tid >> 4; ct < nc * 9; ct += blockDim.x >> 4)
+                    wsm[ct * n8 + c] = ci0 + c < cin ? __bfloat162float(wsrc[size_t(ct) * cin + c]) : 0.f;
         }
         __syncthreads();
         const float* zp = zs + (slot0 * DG_CO + sp) * ZS + 4 + 4 * xt;
         const float* wp = wsm + sp * 9 * n8 + 4 * cib;
 #pragma unroll 1
-        for (int co = sp; co < nc; co += d.S, zp += d.S * ZS, wp += d.S * 9 * n8) {
+        for (int co = sp < d.S ? sp : nc; co < nc; co += d.S, zp += d.S * ZS, wp += d.S * 9 * n8) {
             u64 z[4][6];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -656,7 +671,7 @@ cudaError_t conv_dgrad(const ConvBwd& L, const float* dZ, const bf16* Wt, int Bn
     auto kern = L.H == 32 ? k_dgrad3<32> : L.H == 16 ? k_dgrad3<16> : L.H == 8 ? k_dgrad3<8> : k_dgrad3<4>;
     const cudaError_t e = raise_smem_limit(kern, d.smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.threads, d.smem, s>>>(dZ, L.cout, Wt, L.ca, L.cb, pairs, d,
+    kern<<<dim3((pairs + d.pairs - 1) / d.pairs, d.ny), d.block, d.smem, s>>>(dZ, L.cout, Wt, L.ca, L.cb, pairs, d,
                                                                                act, dIn, lo, lo_act);
     return cudaGetLastError();
 }
