@@ -567,6 +567,14 @@ static bool takes_fused(const fwr_plan* p, int iters) {
     return fwr::fused_supported(p->N, 4, p->n) || (p->periodic == FWR_PERIODIC_BEFORE_EACH_FFT && iters >= 2);
 }
 
+// whether a cluster launch found no room for a cluster (a context with few of
+// the SMs): one CTA per frame needs none
+static bool no_clusters(cudaError_t e) {
+    if (e != cudaErrorInvalidConfiguration && e != cudaErrorLaunchOutOfResources) return false;
+    cudaGetLastError();
+    return true;
+}
+
 fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext_init, int n_frames, int iters,
                               float* phase, float* ext_out, void* stream) {
     fwr_status st = check_call(p, slopes, n_frames, iters, phase, ext_out);
@@ -612,14 +620,17 @@ fwr_status fwr_reconstruct_ex(fwr_plan* p, const float* slopes, const float* ext
     } else if (p->N >= 256) {
         if (ext_out || !phase) return FWR_ERR_UNSUPPORTED;
         e = fwr::launch_slab(p->N, k, p->d_scratch, p->d_counters, p->scratch_ctas, static_cast<cudaStream_t>(stream));
-    } else if (p->N == 128 && phase && !ext_out && !p->one_cta(n_frames) && takes_fused(p, iters) &&
-               fwr::cluster128_wanted(n_frames, p->sms)) {
-        // few frames on every SM (no FWR_OPT_CTAS of the caller's); pupils that
-        // the fused kernel takes, whose bits these are
-        e = fwr::launch_cluster_f32(k, p->sms, static_cast<cudaStream_t>(stream));
+    } else if (takes_fused(p, iters)) {
+        // few frames on every SM (no FWR_OPT_CTAS of the caller's): the same bits
+        bool shared = p->N == 128 && phase && !ext_out && !p->one_cta(n_frames) &&
+                      fwr::cluster128_wanted(n_frames, p->sms);
+        if (shared) {
+            e = fwr::launch_cluster_f32(k, p->sms, static_cast<cudaStream_t>(stream));
+            shared = !no_clusters(e);
+        }
+        if (!shared) e = fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream));
     } else {
-        e = takes_fused(p, iters) ? fwr::launch_fused_f32(p->N, k, static_cast<cudaStream_t>(stream))
-                                  : fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
+        e = fwr::launch_basic_f32(p->N, k, static_cast<cudaStream_t>(stream));
     }
     return e == cudaSuccess ? FWR_OK : cuda_fail(e, "gerchberg launch");
 }
@@ -708,13 +719,20 @@ fwr_status fwr_reconstruct_f64(fwr_plan* p, const double* slopes, const double* 
         if (!pow2(p->N) || !fwr::fused_supported(p->N, 8, p->n)) return FWR_ERR_UNSUPPORTED;
         k.hud = p->d_hud;
     }
-    cudaError_t e = !pow2(p->N) ? fwr::launch_anygrid_f64(p->N, k, static_cast<cudaStream_t>(stream))
-                    // few frames on every SM (no FWR_OPT_CTAS of the caller's)
-                    : phase && !ext_out && !p->one_cta(n_frames) && fwr::cluster64_wanted(p->N, n_frames, p->sms)
-                        ? fwr::launch_cluster_f64(p->N, k, static_cast<cudaStream_t>(stream))
-                    : fwr::fused_supported(p->N, 8, p->n)
-                        ? fwr::launch_fused_f64(p->N, k, static_cast<cudaStream_t>(stream))
-                        : fwr::launch_basic_f64(p->N, k, static_cast<cudaStream_t>(stream));
+    cudaError_t e = cudaSuccess;
+    if (!pow2(p->N)) {
+        e = fwr::launch_anygrid_f64(p->N, k, static_cast<cudaStream_t>(stream));
+    } else {
+        // few frames on every SM (no FWR_OPT_CTAS of the caller's)
+        bool shared = phase && !ext_out && !p->one_cta(n_frames) && fwr::cluster64_wanted(p->N, n_frames, p->sms);
+        if (shared) {
+            e = fwr::launch_cluster_f64(p->N, k, static_cast<cudaStream_t>(stream));
+            shared = !no_clusters(e);
+        }
+        if (!shared)
+            e = fwr::fused_supported(p->N, 8, p->n) ? fwr::launch_fused_f64(p->N, k, static_cast<cudaStream_t>(stream))
+                                                    : fwr::launch_basic_f64(p->N, k, static_cast<cudaStream_t>(stream));
+    }
     return e == cudaSuccess ? FWR_OK : cuda_fail(e, "gerchberg f64 launch");
 }
 
@@ -901,8 +919,10 @@ cudaError_t fwr::launch_warm_bf16(fwr_plan* p, const float* slopes, const uint16
     k.shape = p->shape;
     k.ctas = p->ctas;
     k.status = p->d_status;
-    if (p->N == 128 && !p->one_cta(n_frames) && fwr::cluster128_wanted(n_frames, p->sms))
-        return fwr::launch_cluster_f32(k, p->sms, s);
+    if (p->N == 128 && !p->one_cta(n_frames) && fwr::cluster128_wanted(n_frames, p->sms)) {
+        const cudaError_t e = fwr::launch_cluster_f32(k, p->sms, s);
+        if (!no_clusters(e)) return e;
+    }
     k.pdl = pdl ? 1 : 0;
     return fwr::launch_fused_f32(p->N, k, s);
 }
