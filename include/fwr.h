@@ -230,8 +230,9 @@ fwr_status fwr_plan_create(fwr_plan** out, int n_lenslets, double pad_factor,
  * the paper's small windows of w lenslets around the pupil (N = n + 2w,
  * Sec. 4.1: w = 3 and 6). N >= n + 2. A power of two in {16, ..., 256} gives
  * the same plan as fwr_plan_create. Any other N must be even and in
- * [16, 64]: such plans run the direct-DFT kernel (every 1-D transform a
- * direct sum over the line, O(N) per output) in FP32 and FP64 through
+ * [16, 64]: such plans run the direct-DFT kernel (every 1-D transform as
+ * folded sums over the line's even and odd elements, about N / 4 products per
+ * real output) in FP32 and FP64 through
  * fwr_reconstruct, _ex, _f64 and _host, with every periodic mode, both
  * filters, warm starts and ext_out; the Hudgin extension, the DFT-as-GEMM
  * transform, ragged batches, the static-scratch call and warm-start objects
